@@ -133,7 +133,7 @@ def _block(B, K, V, dtype, seed):
     return z.view(B, K + 1, V), _drafts(g, B, K, V, at[:, :K, 0], at[:, :K, 1])
 
 
-def _head(B, K, V, H, seed, lo=0, hi=None):
+def _head(B, K, V, H, seed):
     """Hidden states [B(K+1), H] and LM-head weight [V, H] (bf16) and drafts: the weight is N(0, 0.02^2), each
     hidden row leans towards two tokens' weight rows, close to each other in a fifth of the rows."""
     g = torch.Generator(device="cuda")
