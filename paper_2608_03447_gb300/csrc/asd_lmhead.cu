@@ -22,12 +22,14 @@
 // CTA's barrier; warp 1 allocates tensor memory, and in the first CTA one of
 // its threads issues the MMAs; warps 2-9 read the two accumulators (192 of the
 // 512 TMEM columns each) with tcgen05.ld, one warp per lane quarter and tile.
-// The epilogue turns each 32 x 32 block (vocabulary rows x token columns) of a
-// warp around through shared memory, so that a lane holds one token column and
-// reduces it with plain register arithmetic, and keeps a running (value, index)
-// key per token. The MMAs of the next unit wait for the epilogue: two
-// accumulators fill the tensor memory, and this costs less than the extra L2
-// traffic of one vocabulary tile per unit with double-buffered accumulators.
+// The epilogue reads each 32 x 32 block (vocabulary rows x token columns) of a
+// warp as matrix fragments, four rows of eight columns per thread, so a column's
+// maximum over a thread's rows is register arithmetic; it goes on to find where
+// a maximum sits only in blocks where some column reaches the best logit that
+// the token has so far (see reduce_block). The MMAs of the next unit wait for
+// the epilogue: two accumulators fill the tensor memory, and this costs less
+// than the extra L2 traffic of one vocabulary tile per unit with
+// double-buffered accumulators.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -51,7 +53,7 @@ constexpr int kBK = 64;                   // K per stage: 64 bf16 = one 128-byte
 constexpr int kUmmaK = 16;                // K per tcgen05.mma (kind::f16)
 constexpr int kW = 2;                     // vocabulary tiles per unit (MMAs per token slab)
 constexpr int kUnitM = kW * kPairM;       // vocabulary rows per pair per unit
-constexpr int kStages = 4;
+constexpr int kStages = 5;                // 220 KB of the 227 KB a CTA may have
 constexpr int kStageB = kHalfN * kBK * 2;  // 12 KB of token rows
 constexpr int kSlabA = kHalfM * kBK * 2;   // 16 KB of vocabulary rows per tile
 constexpr int kStageA = kW * kSlabA;
@@ -61,7 +63,6 @@ constexpr int kLmThreads = (2 + kEpiWarps) * 32;  // producer, MMA, epilogue war
 constexpr int kTmemCols = 512;            // accumulator j at column j * 256
 constexpr int kAccStride = 256;
 constexpr int kChunks = kTN / 32;         // 32-column TMEM loads per accumulator
-constexpr int kPitch = 36;                // floats per row of an epilogue transpose block (conflict-free)
 static_assert(kTN % 32 == 0 && kHalfN % 8 == 0, "token tile: whole 32-column loads, whole 8-row swizzle groups");
 static_assert((kW - 1) * kAccStride + kTN <= kTmemCols, "accumulators fit in tensor memory");
 
@@ -74,7 +75,8 @@ struct LmShared {
   uint32_t tmem_base;
   int abort;
   int draft[kTN];                     // x of the tile's token rows (-1: no draft / out of range)
-  alignas(16) float xpose[kEpiWarps][32 * kPitch];  // per epilogue warp: a 32 x 32 block turned around
+  alignas(16) float thr[kTN];         // each token's best logit when the unit began: less cannot win
+  unsigned long long best[kTN];       // each token's best (value, index) key, as far as this CTA knows
 };
 // dynamic shared memory: [1 KB alignment slack][stages x B][stages x A][LmShared]
 constexpr size_t kLmSmemBytes = 1024 + static_cast<size_t>(kStages) * (kStageA + kStageB) + sizeof(LmShared);
@@ -202,6 +204,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
+// Rows l / 4 and l / 4 + 8 (of 16 TMEM lanes from the one addressed on) of lane
+// l's warp, 32 consecutive fp32 columns: r[4g + e] is row l / 4, r[4g + 2 + e]
+// row l / 4 + 8, both of column 8g + 2 (l % 4) + e.
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // The sticky error word, when the call has a workspace (asd_lmhead_logits has none).
@@ -218,6 +231,112 @@ __device__ __forceinline__ void abort_pair(LmShared& sh, uint32_t peer) {
 // Order-preserving bits of a column maximum; NaN is mapped above +inf
 // whatever its sign bit, so a NaN anywhere in a row reaches the row's key.
 __device__ __forceinline__ uint32_t max_bits(float v) { return v != v ? 0xffc00000u : ordered_bits(v); }
+
+// Meets the kThreads threads of the epilogue warps.
+__device__ __forceinline__ void epilogue_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+}
+
+// Argmax of one warp's 32 x 32 block of logits: vocabulary rows v_warp on (TMEM
+// lanes lane_base on) by token columns c on of the tile.
+//
+// What this costs is the time the tensor cores wait for it, so the common case
+// is kept short: as fragments, a thread holds rows l/4 + {0, 8, 16, 24} of eight
+// columns, three maxima a column with no other lane needed, and one vote tells
+// whether any column of the block reaches its token's best logit so far. Once
+// the first units are in, that is rare (a block of 32 of the V rows holds the
+// best of all rows so far for a token), and only then the lanes exchange maxima
+// (seven shuffles leave one column per lane) and look for the lowest row that
+// holds them. Turning the block around through shared memory instead, which
+// gives every column's index every time, took about 520 cycles a block with
+// eight warps at it, and 36 KB that now hold a fifth stage of the ring. Back to
+// back under the power cap: 604 -> 597 us for 576 tokens (624 against 658 us
+// for a first pass), 2159 -> 2134 us for 2304, 90.8 -> 85.7 us for 160 tokens on
+// a 37984-row shard. A NaN passes the vote and reaches the token's key.
+__device__ __forceinline__ void reduce_block(LmShared& sh, const VerifyParams& p, uint32_t tmem_block, int c,
+                                             int tok0, int T, int v_warp, int lane) {
+  uint32_t r[2][16];
+  tmem_ld_frag(tmem_block, r[0]);
+  tmem_ld_frag(tmem_block + (16u << 16), r[1]);
+  const int q = lane >> 2, j = lane & 3;
+  float2 thr[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) thr[g] = *reinterpret_cast<const float2*>(&sh.thr[c + 8 * g + 2 * j]);
+  const int x = sh.draft[c + lane] - v_warp;  // lane l: the row of column c + l's draft token
+  tmem_ld_wait();
+
+  // draft logits: the thread holding row x of column i keeps z_i(x) (rare: at most one row per column)
+  unsigned hit = __ballot_sync(kFull, static_cast<unsigned>(x) < 32u);
+  while (hit) {
+    const int i = __ffs(hit) - 1;
+    hit &= hit - 1;
+    const int row = __shfl_sync(kFull, x, i);
+    if (q == (row & 7) && j == ((i & 7) >> 1)) {
+      const int at = 4 * (i >> 3) + 2 * ((row >> 3) & 1) + (i & 1);
+      float z = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (k == at) z = __uint_as_float(row & 16 ? r[1][k] : r[0][k]);
+      p.draft_logit[tok0 + c + i] = z;
+    }
+  }
+  if (v_warp + 31 >= p.V) {  // the last, partial tile: rows past V never win
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (v_warp + 16 * h + 8 * ((k >> 1) & 1) + q >= p.V) r[h][k] = __float_as_uint(-INFINITY);
+  }
+
+  float m[8];  // column 8 (i / 2) + 2j + i % 2: the maximum of this thread's four rows
+  bool reaches = false;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = 4 * (i >> 1) + (i & 1);
+    m[i] = fmax_nan(fmax_nan(__uint_as_float(r[0][k]), __uint_as_float(r[0][k + 2])),
+                    fmax_nan(__uint_as_float(r[1][k]), __uint_as_float(r[1][k + 2])));
+    reaches |= !(m[i] < (i & 1 ? thr[i >> 1].y : thr[i >> 1].x));
+  }
+  if (!__any_sync(kFull, reaches)) return;
+
+  // One column per lane: of its columns a lane keeps those whose index bit
+  // equals its own bit, and hands the others over.
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  float m4[4], m2[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    m4[i] = fmax_nan(b4 ? m[i + 4] : m[i], __shfl_xor_sync(kFull, b4 ? m[i] : m[i + 4], 16));
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    m2[i] = fmax_nan(b3 ? m4[i + 2] : m4[i], __shfl_xor_sync(kFull, b3 ? m4[i] : m4[i + 2], 8));
+  const float zmax = fmax_nan(b2 ? m2[1] : m2[0], __shfl_xor_sync(kFull, b2 ? m2[0] : m2[1], 4));
+  const int mine = c + ((lane >> 3) & 3) * 8 + 2 * j + ((lane >> 2) & 1);
+  const uint32_t hi = max_bits(zmax);
+  const bool wins = tok0 + mine < T && hi >= static_cast<uint32_t>(sh.best[mine] >> 32);
+  if (!__any_sync(kFull, wins)) return;
+
+  // the lowest row that holds each column's maximum; none does for a NaN
+  int w[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float z = __shfl_sync(kFull, zmax, (i << 2) | j);
+    const int k = 4 * (i >> 1) + (i & 1);
+    w[i] = __uint_as_float(r[0][k]) == z       ? q
+           : __uint_as_float(r[0][k + 2]) == z ? q + 8
+           : __uint_as_float(r[1][k]) == z     ? q + 16
+           : __uint_as_float(r[1][k + 2]) == z ? q + 24
+                                               : 32;
+  }
+  int w4[4], w2[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w4[i] = min(b4 ? w[i + 4] : w[i], __shfl_xor_sync(kFull, b4 ? w[i] : w[i + 4], 16));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) w2[i] = min(b3 ? w4[i + 2] : w4[i], __shfl_xor_sync(kFull, b3 ? w4[i] : w4[i + 2], 8));
+  const int row = min(b2 ? w2[1] : w2[0], __shfl_xor_sync(kFull, b2 ? w2[0] : w2[1], 4)) & 31;
+  if (wins)
+    atomicMax(&sh.best[mine], (static_cast<unsigned long long>(hi) << 32) |
+                                  (0xffffffffu - static_cast<uint32_t>(v_warp + row)));
+}
 
 struct LmParams {
   int T, H, V;
@@ -367,97 +486,64 @@ __global__ void __launch_bounds__(kLmThreads, 1)
     const int jt = (warp - 2) >> 2;                   // the unit's vocabulary tile this warp reduces
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const uint32_t acc_empty0 = map_rank(smem_u32(&sh.acc_empty), 0);
-    float* xpose = sh.xpose[warp - 2];
-    int xs[kChunks];  // lane l: draft of token column c * 32 + l
-#pragma unroll
-    for (int c = 0; c < kChunks; ++c) xs[c] = kWriteLogits ? -1 : sh.draft[c * 32 + lane];
-    unsigned long long best[kChunks];  // lane l: running key of token column c * 32 + l
-#pragma unroll
-    for (int c = 0; c < kChunks; ++c) best[c] = 0ull;
+    const int et = static_cast<int>(threadIdx.x) - 64;  // this thread among the epilogue's: its token column
+    const int et_tok = m * kTN + et;
+    bool ok = true;
     for (int t = 0; t < n_tiles; ++t) {
-      const bool ok = __all_sync(kFull, mbar_wait_cluster(&sh.acc_full, t & 1, &sh.abort));
-      if (!ok) {
-        if (lane == 0) {
+      const int v_warp = (n_first + t * q.pairs_per_tile) * kUnitM + static_cast<int>(rank) * kW * kHalfM +
+                         jt * kHalfM + quarter * 32;
+      // While the MMAs of the unit run: what each token has to beat, over all CTAs so far
+      unsigned long long known = 0ull;
+      if (!kWriteLogits) {
+        if (et < kTN) {
+          if (et_tok < q.T) known = __ldcg(&p.row_key[et_tok]);
+          sh.best[et] = known;
+          sh.thr[et] = et_tok >= q.T ? INFINITY : known ? ordered_value(static_cast<uint32_t>(known >> 32)) : -INFINITY;
+        }
+        epilogue_sync();
+      }
+      // after a wait that gave up the warp goes on without reducing: the other warps meet it at the barriers
+      if (ok) {
+        ok = __all_sync(kFull, mbar_wait_cluster(&sh.acc_full, t & 1, &sh.abort));
+        if (!ok && lane == 0) {
           abort_pair(sh, peer);
           report_timeout(p);
         }
-        break;
       }
-      tc_fence_after();
-      const int v_warp = (n_first + t * q.pairs_per_tile) * kUnitM + static_cast<int>(rank) * kW * kHalfM +
-                         jt * kHalfM + quarter * 32;
-      const int v = v_warp + lane;  // this thread's vocabulary row
-#pragma unroll
-      for (int c = 0; c < kChunks; ++c) {
-        uint32_t r[32];
-        tmem_ld32(tmem + lane_base + static_cast<uint32_t>(jt * kAccStride + c * 32), r);
-        tmem_ld_wait();
+      if (ok) {
+        tc_fence_after();
+        const uint32_t acc = tmem + lane_base + static_cast<uint32_t>(jt * kAccStride);
         if (kWriteLogits) {
-          if (v < q.V) {
+          const int v = v_warp + lane;  // this thread's vocabulary row
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const int tok = m * kTN + c * 32 + i;
-              if (tok < q.T) q.logits_out[static_cast<long long>(tok) * q.V + v] = __uint_as_float(r[i]);
+          for (int c = 0; c < kChunks; ++c) {
+            uint32_t r[32];
+            tmem_ld32(acc + static_cast<uint32_t>(c * 32), r);
+            tmem_ld_wait();
+            if (v < q.V) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) {
+                const int tok = m * kTN + c * 32 + i;
+                if (tok < q.T) q.logits_out[static_cast<long long>(tok) * q.V + v] = __uint_as_float(r[i]);
+              }
             }
           }
-        } else {
-          // draft logits: the lane holding row x of column i keeps z_i(x) (rare: at most one row per column)
-          unsigned hit = __ballot_sync(kFull, static_cast<unsigned>(xs[c] - v_warp) < 32u);
-          while (hit) {
-            const int i = __ffs(hit) - 1;
-            hit &= hit - 1;
-            const int owner = __shfl_sync(kFull, xs[c], i) - v_warp;
-            if (lane == owner) {
-              float z = 0.0f;
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (j == i) z = __uint_as_float(r[j]);
-              p.draft_logit[m * kTN + c * 32 + i] = z;
-            }
-          }
-          // argmax of each column over the warp's 32 rows: the block is turned
-          // around through shared memory (lane l writes its row, then reads
-          // column l), the lane takes the column's maximum, and where that
-          // raises the column's running key, the lowest row holding it.
-          if (v_warp >= q.V) continue;  // rows past the vocabulary: nothing to reduce
-          if (v_warp + 31 >= q.V && v >= q.V) {  // the last, partial tile: rows past V never win
-#pragma unroll
-            for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(-INFINITY);
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<uint4*>(xpose + lane * kPitch + 4 * i) =
-                make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-          __syncwarp();
-          float col[32];  // column `lane` of the block: the logits of token c * 32 + lane in the warp's 32 rows
-#pragma unroll
-          for (int i = 0; i < 32; ++i) col[i] = xpose[i * kPitch + lane];
-          __syncwarp();  // the block is read before the next chunk overwrites it
-          float zmax = col[0];
-#pragma unroll
-          for (int i = 1; i < 32; ++i) zmax = fmax_nan(zmax, col[i]);
-          const uint32_t hi = max_bits(zmax);
-          if (hi > static_cast<uint32_t>(best[c] >> 32)) {
-            int w = 0;  // NaN: no row compares equal; the key still says NaN
-#pragma unroll
-            for (int i = 31; i >= 0; --i)
-              if (col[i] == zmax) w = i;
-            best[c] = (static_cast<unsigned long long>(hi) << 32) | (0xffffffffu - static_cast<uint32_t>(v_warp + w));
-          }
+        } else if (v_warp < q.V) {  // rows past the vocabulary: nothing to reduce
+          for (int c = 0; c < kTN; c += 32)
+            reduce_block(sh, p, acc + static_cast<uint32_t>(c), c, m * kTN, q.T, v_warp, lane);
         }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_remote(acc_empty0);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_remote(acc_empty0);
-    }
-    if (!kWriteLogits && !sh.abort) {
-#pragma unroll
-      for (int c = 0; c < kChunks; ++c) {
-        const int tok = m * kTN + c * 32 + lane;
-        const unsigned long long key = best[c];
-        if (tok < q.T && key) {
-          atomicMax(&p.row_key[tok], key);
-          if ((key >> 32) == 0xffc00000ull) atomicOr(&p.flags[tok / K1], ASD_STATUS_NAN_LOGIT);
+      if (!kWriteLogits) {
+        epilogue_sync();  // every warp's maxima are in sh.best
+        if (et < kTN && et_tok < q.T) {
+          const unsigned long long key = sh.best[et];
+          if (key != known) {
+            atomicMax(&p.row_key[et_tok], key);
+            if ((key >> 32) == 0xffc00000ull) atomicOr(&p.flags[et_tok / K1], ASD_STATUS_NAN_LOGIT);
+          }
         }
       }
     }
