@@ -192,9 +192,10 @@ int asd_verify_strict(const void* logits, int dtype, int B, int K, int V, const 
  * order, so ties and near-ties (within about 1e-5 of the row's scale) may
  * resolve differently from an exact (fp64) evaluation; exact ties between
  * equal fp32 logits go to the lowest index, as in asd_verify.
- * Launch: clusters of two CTAs, one per SM of a pair, each with about 214 KB
+ * Launch: clusters of two CTAs, one per SM of a pair, each with up to 227 KB
  * of shared memory and all 512 tensor-memory columns of its SM, so a call
- * occupies the GPU's SM pairs while it runs.
+ * occupies the GPU's SM pairs while it runs; the selection runs in a small
+ * kernel right behind.
  */
 int asd_lmhead_workspace_size(int B, int K, int V, int H, size_t* bytes);
 int asd_lmhead_verify(const void* hidden, const void* weight, int H, int B, int K, int V,

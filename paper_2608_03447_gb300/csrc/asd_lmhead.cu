@@ -9,27 +9,27 @@
 //
 // Tiling: two CTAs on a pair of SMs (a cluster of 2) share 2-SM MMAs
 // (tcgen05 cta_group::2). An MMA's M is 256 vocabulary rows (128 per SM: the
-// TMEM lanes), its N is 192 token rows (the TMEM columns), and the 576 rows of
-// a B = 64, K = 8 step are exactly three token tiles (no padded rows). A pair
-// works in units of two vocabulary tiles (512 rows) against one token tile:
-// per 64-deep K step each SM loads 256 rows of W and half (96) of the token
-// rows, 44 KB, and issues two MMAs over the same token slab, so the token rows
-// cross from L2 once per two vocabulary tiles. A pair owns one token tile and
-// walks the units with a stride; the pairs of the three token tiles that share
-// a unit run at the same time, so each W tile comes from HBM once and from L2
-// for the other two. Per CTA: warp 0 issues TMA loads (128B-swizzled 64-wide K
-// slabs) into a kStages-deep ring, whose completion is counted on the first
-// CTA's barrier; warp 1 allocates tensor memory, and in the first CTA one of
-// its threads issues the MMAs; warps 2-9 read the two accumulators (192 of the
-// 512 TMEM columns each) with tcgen05.ld, one warp per lane quarter and tile.
+// TMEM lanes), its N is one token tile (the TMEM columns): the T token rows are
+// cut into as few tiles of at most 256 columns as hold them, all of the same
+// width (T = 576: three of 192, no padding; T = 18: one of 32). A pair works
+// through items of two vocabulary tiles (512 rows) by one token tile: per
+// 64-deep K step each SM loads 2 x 128 rows of W and half of the token rows and
+// issues two MMAs per K slice over the same token slab, so the token rows cross
+// from L2 once per two vocabulary tiles. Items are dealt to the pairs in one
+// sequence, token tiles innermost, so the pairs that need a W row run at the
+// same time and it comes from HBM about once (see LmParams for the last round).
+// Per CTA: warp 0 issues TMA loads (128B-swizzled 64-wide K slabs) into a ring
+// of as many stages as fit, whose completion is counted on the first CTA's
+// barrier; warp 1 allocates tensor memory, and in the first CTA one of its
+// threads issues the MMAs; warps 2-9 reduce the accumulators. Accumulators are
+// slots in a ring of two to four (512 columns / token tile width), each handed
+// over by barriers of its own, so that the MMAs of the next item begin when one
+// tile has been read and run ahead in it while the other is being read.
 // The epilogue reads each 32 x 32 block (vocabulary rows x token columns) of a
 // warp as matrix fragments, four rows of eight columns per thread, so a column's
 // maximum over a thread's rows is register arithmetic; it goes on to find where
 // a maximum sits only in blocks where some column reaches the best logit that
-// the token has so far (see reduce_block). The MMAs of the next unit wait for
-// the epilogue: two accumulators fill the tensor memory, and this costs less
-// than the extra L2 traffic of one vocabulary tile per unit with
-// double-buffered accumulators.
+// the token has so far (see reduce_block).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -40,6 +40,7 @@
 
 #include "asd.h"
 #include "asd_device.cuh"
+#include "asd_select.cuh"
 
 namespace {
 
@@ -47,40 +48,41 @@ using namespace asd_detail;
 
 constexpr int kPairM = 256;               // vocabulary rows per CTA pair in one MMA (MMA M)
 constexpr int kHalfM = 128;               // vocabulary rows per CTA in one MMA (TMEM lanes)
-constexpr int kTN = 192;                  // token rows per tile (MMA N)
-constexpr int kHalfN = kTN / 2;           // token rows each CTA of the pair loads
+constexpr int kMaxTN = 256;               // most token rows per tile (MMA N; a multiple of 32)
 constexpr int kBK = 64;                   // K per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int kUmmaK = 16;                // K per tcgen05.mma (kind::f16)
-constexpr int kW = 2;                     // vocabulary tiles per unit (MMAs per token slab)
-constexpr int kUnitM = kW * kPairM;       // vocabulary rows per pair per unit
-constexpr int kStages = 5;                // 220 KB of the 227 KB a CTA may have
-constexpr int kStageB = kHalfN * kBK * 2;  // 12 KB of token rows
-constexpr int kSlabA = kHalfM * kBK * 2;   // 16 KB of vocabulary rows per tile
+constexpr int kW = 2;                     // vocabulary tiles per item (MMAs per token slab)
+constexpr int kUnitM = kW * kPairM;       // vocabulary rows per item
+constexpr int kMaxStages = 6;
+constexpr int kSlabA = kHalfM * kBK * 2;  // 16 KB of vocabulary rows per tile
 constexpr int kStageA = kW * kSlabA;
-constexpr uint32_t kStageTx = 2u * (kStageA + kStageB);  // both CTAs' bytes, counted on the first CTA
-constexpr int kEpiWarps = 4 * kW;         // one per TMEM lane quarter and vocabulary tile
+constexpr int kMaxSlots = 4;              // accumulators in tensor memory
+constexpr int kEpiWarps = 8;              // two per TMEM lane quarter, 32-column blocks alternating
 constexpr int kLmThreads = (2 + kEpiWarps) * 32;  // producer, MMA, epilogue warps
-constexpr int kTmemCols = 512;            // accumulator j at column j * 256
-constexpr int kAccStride = 256;
-constexpr int kChunks = kTN / 32;         // 32-column TMEM loads per accumulator
-static_assert(kTN % 32 == 0 && kHalfN % 8 == 0, "token tile: whole 32-column loads, whole 8-row swizzle groups");
-static_assert((kW - 1) * kAccStride + kTN <= kTmemCols, "accumulators fit in tensor memory");
+constexpr int kTmemCols = 512;
+static_assert(kEpiWarps * 32 >= kMaxTN, "one epilogue thread per token column");
 
 struct LmShared {
-  unsigned long long full[kStages];   // first CTA: both CTAs' loads of a stage have landed
-  unsigned long long empty[kStages];  // each CTA: the MMAs have read its part of a stage
-  unsigned long long acc_full;        // each CTA: the unit's accumulators are complete
-  unsigned long long acc_empty;       // first CTA: both CTAs' epilogues have read them
+  unsigned long long full[kMaxStages];   // first CTA: both CTAs' loads of a stage have landed
+  unsigned long long empty[kMaxStages];  // each CTA: the MMAs have read its part of a stage
+  unsigned long long acc_full[kMaxSlots];   // each CTA: the slot's accumulator is complete
+  unsigned long long acc_empty[kMaxSlots];  // first CTA: both CTAs' epilogues have read it
   unsigned long long drain;
   uint32_t tmem_base;
   int abort;
-  int draft[kTN];                     // x of the tile's token rows (-1: no draft / out of range)
-  alignas(16) float thr[kTN];         // each token's best logit when the unit began: less cannot win
-  unsigned long long best[kTN];       // each token's best (value, index) key, as far as this CTA knows
+  int draft[kMaxTN];                  // x of the tile's token rows (-1: no draft / out of range)
+  alignas(16) float thr[kMaxTN];      // each token's best logit when the item began: less cannot win
+  unsigned long long best[kMaxTN];    // each token's best (value, index) key, as far as this CTA knows
 };
 // dynamic shared memory: [1 KB alignment slack][stages x B][stages x A][LmShared]
-constexpr size_t kLmSmemBytes = 1024 + static_cast<size_t>(kStages) * (kStageA + kStageB) + sizeof(LmShared);
-static_assert(kLmSmemBytes <= 232448, "shared memory per CTA");
+constexpr size_t kLmSmemMax = 232448;
+constexpr size_t lm_stage_bytes(int tn) { return kStageA + static_cast<size_t>(tn) / 2 * kBK * 2; }
+constexpr int lm_stages(int tn) {
+  const size_t fit = (kLmSmemMax - 1024 - sizeof(LmShared)) / lm_stage_bytes(tn);
+  return fit < kMaxStages ? static_cast<int>(fit) : kMaxStages;
+}
+constexpr size_t lm_smem_bytes(int tn) { return 1024 + lm_stages(tn) * lm_stage_bytes(tn) + sizeof(LmShared); }
+static_assert(lm_stages(192) == 5 && lm_stages(kMaxTN) == 4, "ring depth at the widths that serve most");
 
 // ---------------------------------------------------------------- tcgen05 / TMA / cluster helpers
 
@@ -97,12 +99,14 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
 }
 
 // Instruction descriptor: kind::f16 with bf16 A and B, fp32 D, both K-major,
-// M = kPairM (across the pair), N = kTN.
-constexpr uint32_t kIdesc = (1u << 4)                               // D format: f32
-                            | (1u << 7)                             // A format: bf16
-                            | (1u << 10)                            // B format: bf16
-                            | (static_cast<uint32_t>(kTN >> 3) << 17)     // N / 8
-                            | (static_cast<uint32_t>(kPairM >> 4) << 24); // M / 16
+// M = kPairM (across the pair), N = the token tile's width.
+__device__ __forceinline__ uint32_t instr_desc(int tn) {
+  return (1u << 4)                                     // D format: f32
+         | (1u << 7)                                   // A format: bf16
+         | (1u << 10)                                  // B format: bf16
+         | (static_cast<uint32_t>(tn >> 3) << 17)      // N / 8
+         | (static_cast<uint32_t>(kPairM >> 4) << 24); // M / 16
+}
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -138,6 +142,18 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(unsigned long long* bar, u
       : "memory");
   return done != 0;
 }
+// Whether the phase with the given parity has completed; never sleeps.
+__device__ __forceinline__ bool mbar_test_cluster(unsigned long long* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
 // mbar_wait for barriers that the other CTA of the pair also signals; the
 // abort flag and the clock are checked every 16 sleeps.
 __device__ inline bool mbar_wait_cluster(unsigned long long* bar, uint32_t parity, volatile int* abort) {
@@ -152,6 +168,41 @@ __device__ inline bool mbar_wait_cluster(unsigned long long* bar, uint32_t parit
   }
 }
 
+// The wait of the two warps that feed the tensor cores: by the whole warp, with
+// one answer for all of it, so that the compiler can keep what the loop around
+// it counts in uniform registers, which the MMA and TMA instructions take their
+// operands from; and with the hardware's own short suspend time, which wakes
+// sooner than a long one (609 -> 600 us for 576 tokens).
+__device__ inline bool mbar_wait_warp(unsigned long long* bar, uint32_t parity, volatile int* abort) {
+  auto completed = [&] {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return __all_sync(kFull, done != 0) != 0;
+  };
+  if (completed()) return true;
+  const unsigned long long t0 = global_ns();
+  for (unsigned it = 1;; ++it) {
+    if (completed()) return true;
+    if ((it & 255u) == 0 && __any_sync(kFull, *abort != 0 || global_ns() - t0 > kWaitLimitNs)) return false;
+  }
+}
+// True in one lane of the warp, the same one every time.
+__device__ __forceinline__ bool elect_lane() {
+  uint32_t one;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(one));
+  return one != 0;
+}
+
 // TMA tile load into this CTA's shared memory whose completion is counted on
 // an mbarrier of either CTA of the pair (cluster address).
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar_cluster, int x,
@@ -163,12 +214,13 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       : "memory");
 }
 
-__device__ __forceinline__ void umma_pair_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_pair_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -340,62 +392,71 @@ __device__ __forceinline__ void reduce_block(LmShared& sh, const VerifyParams& p
 
 struct LmParams {
   int T, H, V;
-  int token_tiles;     // ceil(T / kTN)
-  int pairs_per_tile;  // CTA pairs that share one token tile
-  int vocab_units;     // ceil(V / kUnitM)
-  int k_steps;         // ceil(H / kBK)
-  float* logits_out;   // [T, V] when writing logits instead of verifying
+  int tn;           // token rows per tile
+  int token_tiles;  // ceil(T / tn)
+  int stages;       // ring stages
+  int slots;        // accumulator slots
+  int k_steps;      // ceil(H / kBK)
+  // Items 0 .. full - 1: item i is vocabulary rows (i / token_tiles) * kUnitM on by token tile i % token_tiles.
+  // When the last round of the deal would leave more than half of the pairs idle, its items are dealt in
+  // halves (one vocabulary tile each): entries full + 2 h and full + 2 h + 1 are the tiles of item full + h.
+  int full, entries;
+  float* logits_out;  // [T, V] when writing logits instead of verifying
 };
 
-// One CTA pair (cluster of 2): token tile m = pair % token_tiles, vocabulary
-// units n = pair / token_tiles + i * pairs_per_tile (rows n * kUnitM on).
-template <bool kStrict, bool kWriteLogits>
+// One entry of the deal.
+struct LmItem {
+  int row0;  // first vocabulary row
+  int kw;    // vocabulary tiles
+  int m;     // token tile
+};
+__device__ __forceinline__ LmItem lm_item(const LmParams& q, int entry) {
+  const int half = entry - q.full;
+  const int item = half < 0 ? entry : q.full + (half >> 1);
+  LmItem it;
+  it.m = item % q.token_tiles;
+  it.row0 = (item / q.token_tiles) * kUnitM + (half < 0 ? 0 : (half & 1) * kPairM);
+  it.kw = half < 0 && it.row0 + kPairM < q.V ? kW : 1;  // no second tile past the vocabulary
+  return it;
+}
+
+// One CTA pair (cluster of 2) works through entries pair, pair + pairs, ...
+template <bool kWriteLogits>
 __global__ void __launch_bounds__(kLmThreads, 1)
     lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w,
-                         const __grid_constant__ VerifyParams p, const LmParams q) {
+                         const __grid_constant__ VerifyParams p, const __grid_constant__ LmParams q) {
   extern __shared__ __align__(1024) unsigned char lm_smem_raw[];
   const uint32_t raw = smem_u32(lm_smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;  // 1024-byte aligned for the 128-byte swizzle
   unsigned char* gbase = lm_smem_raw + (base - raw);
-  const uint32_t sB = base;                                        // kStages x kStageB
-  const uint32_t sA = base + kStages * kStageB;                    // kStages x kStageA
-  LmShared& sh = *reinterpret_cast<LmShared*>(gbase + kStages * (kStageA + kStageB));
+  const int stages = q.stages;
+  const uint32_t stage_b = static_cast<uint32_t>(q.tn) / 2 * kBK * 2;  // this CTA's half of the token rows
+  const uint32_t sB = base;                                            // stages x stage_b
+  const uint32_t sA = base + static_cast<uint32_t>(stages) * stage_b;  // stages x kStageA
+  LmShared& sh = *reinterpret_cast<LmShared*>(gbase + static_cast<uint32_t>(stages) * (kStageA + stage_b));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(kFull, static_cast<int>(threadIdx.x >> 5), 0);  // uniform, to the compiler too
+  const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank() & 1u;
   const uint32_t peer = rank ^ 1u;
   const bool leader = rank == 0;
-  const int pair = static_cast<int>(blockIdx.x >> 1);
-  const int m = pair % q.token_tiles;
-  const int n_first = pair / q.token_tiles;
-  const int n_tiles =
-      n_first < q.vocab_units ? (q.vocab_units - n_first + q.pairs_per_tile - 1) / q.pairs_per_tile : 0;
+  const int pair = static_cast<int>(blockIdx.x >> 1), pairs = static_cast<int>(gridDim.x >> 1);
   const int K1 = p.K + 1;
 
+  pdl_signal_dependents();  // the selection's CTAs may take their places beside this kernel's
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(&sh.full[s], 1);
       mbar_init(&sh.empty[s], 1);
     }
-    mbar_init(&sh.acc_full, 1);
-    mbar_init(&sh.acc_empty, 2 * kEpiWarps);  // the epilogue warps of both CTAs
+    for (int s = 0; s < kMaxSlots; ++s) {
+      mbar_init(&sh.acc_full[s], 1);
+      mbar_init(&sh.acc_empty[s], 2 * kEpiWarps);  // the epilogue warps of both CTAs
+    }
     mbar_init(&sh.drain, 1);
     sh.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (!kWriteLogits) {
-    for (int c = threadIdx.x; c < kTN; c += kLmThreads) {
-      const int tok = m * kTN + c;
-      int x = -1;
-      if (tok < q.T && (tok % K1) < p.K) {
-        // the row of this CTA's weight that holds the draft token (a vocabulary
-        // shard starts at global index v_offset), if any
-        x = __ldg(p.draft + static_cast<long long>(tok / K1) * p.K + (tok % K1)) - p.v_offset;
-        if (x < 0 || x >= p.V) x = -1;
-      }
-      sh.draft[c] = x;
-    }
   }
   if (warp == 1) {  // tensor memory of both SMs, allocated together by one warp of each CTA
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -406,158 +467,244 @@ __global__ void __launch_bounds__(kLmThreads, 1)
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers exist before either signals the other's
   tc_fence_after();
-  const uint32_t tmem = sh.tmem_base;
+  const uint32_t tmem = __reduce_max_sync(kFull, sh.tmem_base);  // uniform, to the compiler too
+  // everything above touches this SM only; the hidden states, drafts, the workspace and the outputs may be the
+  // previous kernel's
+  pdl_wait_prerequisites();
 
-  int it_issued = 0;
+  int issued = 0, issued_stage = 0;  // producer: loads issued, and the stage the next one goes to
+  uint32_t issued_phase = 0;
+  // The producer and the MMA warp run their loops as whole warps and let one lane issue: counters, descriptors
+  // and coordinates stay in uniform registers. With one thread in the loop each MMA waited for its operands to
+  // be moved there: 576 tokens (three tiles of 192 columns) took as long per item as 256 columns do, 645 us a
+  // call against 525 us with all else equal.
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs; completion counted on the first CTA's barrier)
-    if (lane == 0) {
+    const bool elected = elect_lane();
+    if (elected) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_h)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
-      const uint32_t full0 = map_rank(smem_u32(&sh.full[0]), 0);
-      int it = 0;
-      for (int t = 0; t < n_tiles && !sh.abort; ++t) {
-        const int n = n_first + t * q.pairs_per_tile;
-        for (int k = 0; k < q.k_steps; ++k, ++it) {
-          const int s = it % kStages;
-          if (!mbar_wait_cluster(&sh.empty[s], ((it / kStages) & 1) ^ 1, &sh.abort)) {
-            abort_pair(sh, peer);
-            report_timeout(p);
-            break;
-          }
-          if (leader) mbar_expect_tx(&sh.full[s], kStageTx);
+    }
+    const uint32_t full0 = map_rank(smem_u32(&sh.full[0]), 0);
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int e = pair; ok && e < q.entries; e += pairs) {
+      const LmItem it = lm_item(q, e);
+      const int tok = it.m * q.tn + static_cast<int>(rank) * (q.tn / 2);
+      const int row = it.row0 + static_cast<int>(rank) * kHalfM;
+      const uint32_t tx = 2u * (static_cast<uint32_t>(it.kw) * kSlabA + stage_b);  // both CTAs' bytes
+      for (int k = 0; k < q.k_steps; ++k) {
+        ok = mbar_wait_warp(&sh.empty[s], ph ^ 1u, &sh.abort);
+        if (!ok) break;
+        if (elected) {
+          if (leader) mbar_expect_tx(&sh.full[s], tx);
           const uint32_t bar = full0 + static_cast<uint32_t>(s * sizeof(unsigned long long));
-          tma_load_2d_pair(sB + s * kStageB, &map_h, bar, k * kBK, m * kTN + static_cast<int>(rank) * kHalfN);
-          // this CTA's 128 rows of both vocabulary tiles of the unit: rows n * 512 + rank * 256 on
-          tma_load_2d_pair(sA + s * kStageA, &map_w, bar, k * kBK, n * kUnitM + static_cast<int>(rank) * kW * kHalfM);
-          it_issued = it + 1;
+          tma_load_2d_pair(sB + s * stage_b, &map_h, bar, k * kBK, tok);
+          // this CTA's 128 rows of each vocabulary tile
+          tma_load_2d_pair(sA + s * kStageA, &map_w, bar, k * kBK, row);
+          if (it.kw == 2) tma_load_2d_pair(sA + s * kStageA + kSlabA, &map_w, bar, k * kBK, row + kPairM);
+        }
+        ++issued;
+        if (++s == stages) {
+          s = 0;
+          ph ^= 1u;
         }
       }
     }
+    if (!ok && elected) {
+      abort_pair(sh, peer);
+      report_timeout(p);
+    }
+    issued_stage = s;
+    issued_phase = ph;
   } else if (warp == 1) {
-    // ---------------- MMA issuer (one thread of the first CTA, for both SMs)
-    if (leader && lane == 0) {
-      int it = 0;
-      for (int t = 0; t < n_tiles && !sh.abort; ++t) {
-        // the epilogues of both CTAs have read the previous unit's accumulators
-        if (!mbar_wait_cluster(&sh.acc_empty, (t & 1) ^ 1, &sh.abort)) {
-          abort_pair(sh, peer);
-          report_timeout(p);
-          break;
+    // ---------------- MMA issuer (one warp of the first CTA, for both SMs)
+    if (leader) {
+      const bool elected = elect_lane();
+      const uint32_t idesc = instr_desc(q.tn);
+      const uint64_t a_desc = smem_desc_sw128(sA), b_desc = smem_desc_sw128(sB);
+      // the MMAs of one K step of vocabulary tile j: stage s into the accumulator at column d
+      auto mma_step = [&](int s, int j, uint32_t d, bool first) {
+        const uint64_t ad = a_desc + static_cast<uint32_t>((s * kStageA + j * kSlabA) >> 4);
+        const uint64_t bd = b_desc + ((static_cast<uint32_t>(s) * stage_b) >> 4);
+#pragma unroll
+        for (int kk = 0; kk < kBK / kUmmaK; ++kk)  // 16 elements (32 bytes, encoded 2) along K inside the swizzle row
+          umma_pair_bf16(d, ad + 2u * kk, bd + 2u * kk, idesc, !first || kk > 0 ? 1u : 0u);
+      };
+      int s0 = 0, s1 = 0;  // the stages the first and the second tile's next K step read
+      uint32_t ph = 0;     // of s0
+      int slot = 0;
+      uint32_t slot_ph = 1;
+      bool ok = true;
+      for (int e = pair; ok && e < q.entries; e += pairs) {
+        const int kw = lm_item(q, e).kw;
+        const int slot0 = slot;
+        const uint32_t d0 = tmem + static_cast<uint32_t>(slot0 * q.tn);
+        ok = mbar_wait_warp(&sh.acc_empty[slot0], slot_ph, &sh.abort);
+        if (!ok) break;
+        if (++slot == q.slots) {
+          slot = 0;
+          slot_ph ^= 1u;
         }
-        tc_fence_after();
-        bool ok = true;
-        for (int k = 0; k < q.k_steps; ++k, ++it) {
-          const int s = it % kStages;
-          if (!mbar_wait_cluster(&sh.full[s], (it / kStages) & 1, &sh.abort)) {
-            ok = false;
-            break;
-          }
+        const int slot1 = slot;
+        const uint32_t ph1 = slot_ph;
+        const uint32_t d1 = tmem + static_cast<uint32_t>(slot1 * q.tn);
+        if (kw == 2 && ++slot == q.slots) {
+          slot = 0;
+          slot_ph ^= 1u;
+        }
+        bool free1 = false;  // the second tile's slot has been read
+        int k1 = 0;          // K steps issued for the second tile
+        for (int k = 0; k < q.k_steps; ++k) {
+          ok = mbar_wait_warp(&sh.full[s0], ph, &sh.abort);
+          if (!ok) break;
           tc_fence_after();
-          const uint64_t bd = smem_desc_sw128(sB + s * kStageB);
-#pragma unroll
-          for (int j = 0; j < kW; ++j) {  // both vocabulary tiles of the unit read the same token slab
-            const uint32_t d = tmem + static_cast<uint32_t>(j * kAccStride);
-            const uint64_t ad = smem_desc_sw128(sA + s * kStageA + j * kSlabA);
-#pragma unroll
-            for (int kk = 0; kk < kBK / kUmmaK; ++kk) {
-              // advance 16 elements (32 bytes, encoded 2) along K inside the swizzle row
-              umma_pair_bf16(d, ad + 2u * kk, bd + 2u * kk, (k > 0 || kk > 0) ? 1u : 0u);
+          const bool last = k == q.k_steps - 1;
+          if (elected) {
+            mma_step(s0, 0, d0, k == 0);
+            if (last) umma_commit_pair(&sh.acc_full[slot0]);
+            if (kw == 1) umma_commit_pair(&sh.empty[s0]);  // frees the stage in both CTAs once these MMAs have read it
+          }
+          if (kw == 1) {
+            if (++s1 == stages) s1 = 0;
+          } else {
+            // while the second tile's slot is still being read, the first tile runs ahead as far as the ring goes
+            if (!free1) {
+              if (last || k - k1 + 1 >= stages) {
+                ok = mbar_wait_warp(&sh.acc_empty[slot1], ph1, &sh.abort);
+                if (!ok) break;
+                free1 = true;
+              } else {
+                free1 = __all_sync(kFull, mbar_test_cluster(&sh.acc_empty[slot1], ph1));
+              }
+              tc_fence_after();
+            }
+            for (; free1 && k1 <= k; ++k1) {
+              if (elected) {
+                mma_step(s1, 1, d1, k1 == 0);
+                umma_commit_pair(&sh.empty[s1]);
+              }
+              if (++s1 == stages) s1 = 0;
             }
           }
-          umma_commit_pair(&sh.empty[s]);  // frees the stage in both CTAs when these MMAs have read it
+          if (++s0 == stages) {
+            s0 = 0;
+            ph ^= 1u;
+          }
         }
+        if (ok && kw == 2 && elected) umma_commit_pair(&sh.acc_full[slot1]);
+      }
+      if (elected) {
         if (!ok) {
           abort_pair(sh, peer);
           report_timeout(p);
-          break;
         }
-        umma_commit_pair(&sh.acc_full);  // the accumulators are complete in both CTAs
+        umma_commit_local(&sh.drain);  // arrives once every MMA issued above has finished
+        const unsigned long long t0 = global_ns();
+        while (!mbar_try_wait(&sh.drain, 0) && global_ns() - t0 < kWaitLimitNs) {
+        }
       }
-      umma_commit_local(&sh.drain);  // arrives once every MMA issued above has finished
-      const unsigned long long t0 = global_ns();
-      while (!mbar_try_wait(&sh.drain, 0) && global_ns() - t0 < kWaitLimitNs) {
-      }
+      __syncwarp();
     }
   } else {
-    // ---------------- epilogue: warps 2 .. 1 + kEpiWarps, one vocabulary row (TMEM lane) per thread;
-    // warps 2-5 read the first vocabulary tile of a unit, warps 6-9 the second
+    // ---------------- epilogue: warps 2-9, one TMEM lane quarter each; the two warps of a quarter take
+    // alternate 32-column blocks of every accumulator
     const int quarter = warp & 3;                     // TMEM lanes this warp may read
-    const int jt = (warp - 2) >> 2;                   // the unit's vocabulary tile this warp reduces
+    const int c_first = ((warp - 2) >> 2) * 32;
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
-    const uint32_t acc_empty0 = map_rank(smem_u32(&sh.acc_empty), 0);
+    const uint32_t acc_empty0 = map_rank(smem_u32(&sh.acc_empty[0]), 0);
     const int et = static_cast<int>(threadIdx.x) - 64;  // this thread among the epilogue's: its token column
-    const int et_tok = m * kTN + et;
+    int slot = 0;
+    uint32_t slot_ph = 0;
     bool ok = true;
-    for (int t = 0; t < n_tiles; ++t) {
-      const int v_warp = (n_first + t * q.pairs_per_tile) * kUnitM + static_cast<int>(rank) * kW * kHalfM +
-                         jt * kHalfM + quarter * 32;
-      // While the MMAs of the unit run: what each token has to beat, over all CTAs so far
+    for (int e = pair; e < q.entries; e += pairs) {
+      const LmItem it = lm_item(q, e);
+      const int tok0 = it.m * q.tn;
+      // While the item's MMAs run: its draft tokens, and what each token has to beat, over all CTAs so far
+      const bool has_token = et < q.tn && tok0 + et < q.T;
       unsigned long long known = 0ull;
       if (!kWriteLogits) {
-        if (et < kTN) {
-          if (et_tok < q.T) known = __ldcg(&p.row_key[et_tok]);
+        if (et < q.tn) {
+          int x = -1;
+          if (has_token) {
+            const int tok = tok0 + et, b = tok / K1, j = tok - b * K1;
+            known = __ldcg(&p.row_key[tok]);
+            // the row of this weight that holds the draft token (a vocabulary shard starts at global index
+            // v_offset), if any
+            if (j < p.K) x = __ldg(p.draft + static_cast<long long>(b) * p.K + j) - p.v_offset;
+            if (x < 0 || x >= p.V) x = -1;
+          }
+          sh.draft[et] = x;
           sh.best[et] = known;
-          sh.thr[et] = et_tok >= q.T ? INFINITY : known ? ordered_value(static_cast<uint32_t>(known >> 32)) : -INFINITY;
+          sh.thr[et] = !has_token ? INFINITY : known ? ordered_value(static_cast<uint32_t>(known >> 32)) : -INFINITY;
         }
         epilogue_sync();
       }
-      // after a wait that gave up the warp goes on without reducing: the other warps meet it at the barriers
-      if (ok) {
-        ok = __all_sync(kFull, mbar_wait_cluster(&sh.acc_full, t & 1, &sh.abort));
-        if (!ok && lane == 0) {
-          abort_pair(sh, peer);
-          report_timeout(p);
+      for (int t = 0; t < it.kw; ++t) {
+        // after a wait that gave up the warp goes on without reducing: the other warps meet it at the barriers
+        if (ok) {
+          ok = __all_sync(kFull, mbar_wait_cluster(&sh.acc_full[slot], slot_ph, &sh.abort));
+          if (!ok && lane == 0) {
+            abort_pair(sh, peer);
+            report_timeout(p);
+          }
         }
-      }
-      if (ok) {
-        tc_fence_after();
-        const uint32_t acc = tmem + lane_base + static_cast<uint32_t>(jt * kAccStride);
-        if (kWriteLogits) {
-          const int v = v_warp + lane;  // this thread's vocabulary row
+        if (ok) {
+          tc_fence_after();
+          const uint32_t acc = tmem + lane_base + static_cast<uint32_t>(slot * q.tn);
+          const int v_warp = it.row0 + t * kPairM + static_cast<int>(rank) * kHalfM + quarter * 32;
+          if (v_warp < q.V) {  // rows past the vocabulary: nothing to reduce
+            for (int c = c_first; c < q.tn; c += 64) {
+              if (kWriteLogits) {
+                const int v = v_warp + lane;  // this thread's vocabulary row
+                uint32_t r[32];
+                tmem_ld32(acc + static_cast<uint32_t>(c), r);
+                tmem_ld_wait();
+                if (v < q.V) {
+                  float* out = q.logits_out + static_cast<long long>(tok0 + c) * q.V + v;
 #pragma unroll
-          for (int c = 0; c < kChunks; ++c) {
-            uint32_t r[32];
-            tmem_ld32(acc + static_cast<uint32_t>(c * 32), r);
-            tmem_ld_wait();
-            if (v < q.V) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                const int tok = m * kTN + c * 32 + i;
-                if (tok < q.T) q.logits_out[static_cast<long long>(tok) * q.V + v] = __uint_as_float(r[i]);
+                  for (int i = 0; i < 32; ++i)
+                    if (tok0 + c + i < q.T) out[static_cast<long long>(i) * q.V] = __uint_as_float(r[i]);
+                }
+              } else {
+                reduce_block(sh, p, acc + static_cast<uint32_t>(c), c, tok0, q.T, v_warp, lane);
               }
             }
           }
-        } else if (v_warp < q.V) {  // rows past the vocabulary: nothing to reduce
-          for (int c = 0; c < kTN; c += 32)
-            reduce_block(sh, p, acc + static_cast<uint32_t>(c), c, m * kTN, q.T, v_warp, lane);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_remote(acc_empty0 + static_cast<uint32_t>(slot * sizeof(unsigned long long)));
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_remote(acc_empty0);
+        if (++slot == q.slots) {
+          slot = 0;
+          slot_ph ^= 1u;
+        }
       }
       if (!kWriteLogits) {
         epilogue_sync();  // every warp's maxima are in sh.best
-        if (et < kTN && et_tok < q.T) {
+        if (has_token) {
           const unsigned long long key = sh.best[et];
           if (key != known) {
-            atomicMax(&p.row_key[et_tok], key);
-            if ((key >> 32) == 0xffc00000ull) atomicOr(&p.flags[et_tok / K1], ASD_STATUS_NAN_LOGIT);
+            atomicMax(&p.row_key[tok0 + et], key);
+            if ((key >> 32) == 0xffc00000ull) atomicOr(&p.flags[(tok0 + et) / K1], ASD_STATUS_NAN_LOGIT);
           }
         }
       }
     }
-    __threadfence();
   }
 
   tc_fence_before();
   __syncthreads();
   if (sh.abort && leader && warp == 0 && lane == 0) {
     // wait (bounded) for the loads still in flight before the pair exits
-    for (int it = it_issued > kStages ? it_issued - kStages : 0; it < it_issued; ++it) {
-      const int s = it % kStages;
+    for (int n = issued < stages ? issued : stages; n > 0; --n) {
+      if (--issued_stage < 0) {
+        issued_stage = stages - 1;
+        issued_phase ^= 1u;
+      }
       const unsigned long long t0 = global_ns();
-      while (!mbar_try_wait_cluster(&sh.full[s], (it / kStages) & 1) && global_ns() - t0 < kWaitLimitNs) {
+      while (!mbar_try_wait_cluster(&sh.full[issued_stage], issued_phase) && global_ns() - t0 < kWaitLimitNs) {
       }
     }
   }
@@ -566,20 +713,6 @@ __global__ void __launch_bounds__(kLmThreads, 1)
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-  }
-  if (kWriteLogits || sh.abort) return;
-
-  // Count this CTA's rows of each request of its token tile; the CTA that
-  // completes a request (every CTA of the tile has counted) runs its selection.
-  const int t0 = m * kTN, t1 = (m + 1) * kTN < q.T ? (m + 1) * kTN : q.T;
-  if (t0 < t1) {
-    const int b_first = t0 / K1, b_last = (t1 - 1) / K1;
-    const unsigned long long total = static_cast<unsigned long long>(K1) * 2ull * q.pairs_per_tile;
-    for (int b = b_first + warp; b <= b_last; b += kLmThreads / 32) {
-      const int r0 = b * K1 > t0 ? b * K1 : t0;
-      const int r1 = (b + 1) * K1 < t1 ? (b + 1) * K1 : t1;
-      finish_request<float, kStrict>(p, b, static_cast<unsigned long long>(r1 - r0), total, lane);
-    }
   }
 }
 
@@ -622,7 +755,7 @@ struct LmDevice {
   int major = 0, minor = 0;
   // CTA pairs resident at once, per kernel instance (0: not set up yet); the
   // set-up is idempotent, so two threads racing to do it store the same value
-  std::atomic<int> pairs[4] = {};
+  std::atomic<int> pairs[2] = {};
 };
 
 int lm_device(LmDevice** out) {
@@ -643,55 +776,82 @@ int lm_device(LmDevice** out) {
   return ASD_OK;
 }
 
-cudaLaunchConfig_t pair_config(unsigned grid, cudaStream_t stream, cudaLaunchAttribute* attr) {
+cudaLaunchConfig_t pair_config(unsigned grid, size_t smem, cudaStream_t stream, cudaLaunchAttribute (&attr)[2],
+                               bool pdl) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(kLmThreads, 1, 1);
-  cfg.dynamicSmemBytes = kLmSmemBytes;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  attr->id = cudaLaunchAttributeClusterDimension;
-  attr->val.clusterDim.x = 2;
-  attr->val.clusterDim.y = 1;
-  attr->val.clusterDim.z = 1;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 2 : 1;
   return cfg;
 }
 
-template <bool kStrict, bool kWriteLogits>
+// How T token rows and V vocabulary rows are cut and dealt to `pairs` CTA pairs.
+//
+// Token tiles: as few as hold T at up to 256 columns (each tile reads W once
+// more from L2, and a wider MMA reads its vocabulary operand from shared memory
+// less often per product), all of one width, rounded up to the 32 columns of an
+// epilogue block. Against a fixed width of 192: 320 rows took 384 columns and
+// take 2 x 160, 18 rows take 32, 2304 rows take 9 tiles instead of 12.
+//
+// The last round of the deal: `left` items for more pairs. Up to half of the
+// pairs' number, half items keep twice as many pairs busy for half the time;
+// beyond that, halves would only begin a second round.
+void lm_plan(int T, int V, int H, int pairs, LmParams* q) {
+  q->T = T;
+  q->H = H;
+  q->V = V;
+  q->token_tiles = (T + kMaxTN - 1) / kMaxTN;
+  const int per = (T + q->token_tiles - 1) / q->token_tiles;
+  q->tn = (per + 31) / 32 * 32;
+  q->stages = lm_stages(q->tn);
+  q->slots = kTmemCols / q->tn < kMaxSlots ? kTmemCols / q->tn : kMaxSlots;
+  q->k_steps = (H + kBK - 1) / kBK;
+  const int items = (V + kUnitM - 1) / kUnitM * q->token_tiles;
+  const int left = items % pairs;
+  const int halved = 2 * left <= pairs ? left : 0;
+  q->full = items - halved;
+  q->entries = items + halved;
+}
+
+template <bool kWriteLogits>
 int launch_lmhead(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
                   cudaStream_t stream) {
   LmDevice* dev = nullptr;
   int rc = lm_device(&dev);
   if (rc != ASD_OK) return rc;
   if (dev->major != 10) return ASD_ERR_DEVICE;  // tcgen05 needs a Blackwell (sm_10x) device
-  auto kernel = lmhead_verify_kernel<kStrict, kWriteLogits>;
-  const int slot = (kStrict ? 1 : 0) + (kWriteLogits ? 2 : 0);
-  cudaLaunchAttribute attr;
-  int pairs = dev->pairs[slot].load(std::memory_order_acquire);
+  auto kernel = lmhead_verify_kernel<kWriteLogits>;
+  std::atomic<int>& resident = dev->pairs[kWriteLogits ? 1 : 0];
+  cudaLaunchAttribute attr[2];
+  int pairs = resident.load(std::memory_order_acquire);
   if (pairs == 0) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemBytes)) !=
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax)) !=
         cudaSuccess)
       return ASD_ERR_CUDA;
-    cudaLaunchConfig_t probe = pair_config(static_cast<unsigned>(dev->sms & ~1), stream, &attr);
+    // every token tile width leaves room for one CTA per SM
+    cudaLaunchConfig_t probe = pair_config(static_cast<unsigned>(dev->sms & ~1), kLmSmemMax, stream, attr, false);
     if (cudaOccupancyMaxActiveClusters(&pairs, kernel, &probe) != cudaSuccess || pairs < 1) return ASD_ERR_CUDA;
-    dev->pairs[slot].store(pairs, std::memory_order_release);
+    resident.store(pairs, std::memory_order_release);
   }
-  CUtensorMap map_h, map_w;
-  if (!make_map(&map_h, hidden, T, H, kHalfN) || !make_map(&map_w, weight, p.V, H, kW * kHalfM)) return ASD_ERR_CUDA;
   LmParams q;
-  q.T = T;
-  q.H = H;
-  q.V = p.V;
-  q.token_tiles = (T + kTN - 1) / kTN;
-  q.pairs_per_tile = pairs / q.token_tiles > 0 ? pairs / q.token_tiles : 1;
-  q.vocab_units = (p.V + kUnitM - 1) / kUnitM;
-  if (q.pairs_per_tile > q.vocab_units) q.pairs_per_tile = q.vocab_units;
-  q.k_steps = (H + kBK - 1) / kBK;
+  lm_plan(T, p.V, H, pairs, &q);
   q.logits_out = logits_out;
-  const unsigned grid = 2u * static_cast<unsigned>(q.token_tiles * q.pairs_per_tile);
-  cudaLaunchConfig_t cfg = pair_config(grid, stream, &attr);
-  return cudaLaunchKernelEx(&cfg, kernel, map_h, map_w, p, q) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+  CUtensorMap map_h, map_w;
+  if (!make_map(&map_h, hidden, T, H, q.tn / 2) || !make_map(&map_w, weight, p.V, H, kHalfM)) return ASD_ERR_CUDA;
+  const unsigned grid = 2u * static_cast<unsigned>(q.entries < pairs ? q.entries : pairs);
+  cudaLaunchConfig_t cfg = pair_config(grid, lm_smem_bytes(q.tn), stream, attr, true);
+  if (cudaLaunchKernelEx(&cfg, kernel, map_h, map_w, p, q) != cudaSuccess) return ASD_ERR_CUDA;
+  if (kWriteLogits) return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+  return launch_select<float, false>(p, true, stream);
 }
 
 int check_lm_inputs(const void* hidden, const void* weight, int H) {
@@ -754,7 +914,7 @@ int asd_lmhead_verify(const void* hidden, const void* weight, int H, int B, int 
   p.error = reinterpret_cast<unsigned int*>(ws + l.error);
   p.row_top = row_top;
   p.nblk = 1;
-  return launch_lmhead<false, false>(hidden, weight, H, B * (K + 1), p, nullptr,
+  return launch_lmhead<false>(hidden, weight, H, B * (K + 1), p, nullptr,
                                      reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -789,7 +949,7 @@ int asd_lmhead_partials(const void* hidden, const void* weight, int H, int B, in
   p.v_offset = v_offset;
   p.v_total = V;
   p.partials = partials;
-  return launch_lmhead<true, false>(hidden, weight, H, B * (K + 1), p, nullptr,
+  return launch_lmhead<false>(hidden, weight, H, B * (K + 1), p, nullptr,
                                     reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -804,7 +964,7 @@ int asd_lmhead_logits(const void* hidden, const void* weight, int H, int T, int 
   p.V = V;
   p.K = 0;
   p.nblk = 1;
-  return launch_lmhead<false, true>(hidden, weight, H, T, p, logits, reinterpret_cast<cudaStream_t>(stream));
+  return launch_lmhead<true>(hidden, weight, H, T, p, logits, reinterpret_cast<cudaStream_t>(stream));
 }
 
 }  // extern "C"

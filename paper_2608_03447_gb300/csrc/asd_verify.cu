@@ -31,6 +31,7 @@
 
 #include "asd.h"
 #include "asd_device.cuh"
+#include "asd_select.cuh"
 
 namespace {
 
@@ -817,27 +818,6 @@ __global__ void __launch_bounds__(kTmaThreads, ASD_TMA_MIN_BLOCKS)
   }
 }
 
-// ---------------------------------------------------------------- split selection kernel
-//
-// With the row stage in verify_tma_kernel<..., kSplit = true>, the selection of
-// every request runs here: one warp per request, launched right behind the row
-// stage (programmatic dependent launch); griddepcontrol.wait returns once the
-// row stage has completed and its writes are visible, so no counters and no
-// fences are needed, and the streaming CTAs leave their SMs as soon as they
-// have merged their rows.
-
-constexpr int kSelectThreads = 128;  // small: fits beside the streaming CTAs on an SM
-
-template <typename T, bool kStrict>
-__global__ void __launch_bounds__(kSelectThreads) select_kernel(const __grid_constant__ VerifyParams p) {
-  pdl_signal_dependents();
-  pdl_wait_prerequisites();
-  const int lane = threadIdx.x & 31;
-  const int warps = kSelectThreads / 32;
-  for (int b = blockIdx.x * warps + (threadIdx.x >> 5); b < p.B; b += gridDim.x * warps)
-    select_request<T, kStrict>(p, b, lane);
-}
-
 // ---------------------------------------------------------------- host side
 
 // Resident warps of a kernel on the current device, queried once per device.
@@ -974,13 +954,7 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
   }
   if (cudaLaunchKernelEx(&cfg, verify_tma_kernel<T, kStrict, true>, p, bulk_end, per_cta) != cudaSuccess)
     return ASD_ERR_CUDA;
-  cudaLaunchConfig_t sel = cfg;
-  constexpr int kWarps = kSelectThreads / 32;
-  sel.gridDim = dim3(static_cast<unsigned>((p.B + kWarps - 1) / kWarps));
-  sel.blockDim = dim3(kSelectThreads);
-  sel.dynamicSmemBytes = 0;
-  if (cudaLaunchKernelEx(&sel, select_kernel<T, kStrict>, p) != cudaSuccess) return ASD_ERR_CUDA;
-  return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+  return launch_select<T, kStrict>(p, opt.pdl, stream);
 }
 
 // Which kernel streams the logits: the TMA pipeline for inputs of at least

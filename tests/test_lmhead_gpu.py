@@ -223,6 +223,32 @@ def test_lmhead_full_size_exact_inputs_bit_exact(asd):
     assert int((o["accepted_len"] > 0).sum()) > 0
 
 
+# Token tiles (T rows in ceil(T / 256) tiles of one width, a multiple of 32) and the deal of 512-row items to the
+# GPU's 76 CTA pairs: one row, a full and a just exceeded 32-column block, the widest tile, two and three tiles with
+# masked columns, three accumulator slots (width 160); a last round of halves (77 items), of halves whose second one
+# lies past the vocabulary, of whole items (76 + 39), and one partial item; one, three and eight K steps.
+@pytest.mark.parametrize("B,K,H,V", [(1, 0, 8, 39424), (4, 7, 136, 39424), (33, 0, 512, 39000), (32, 7, 136, 39040),
+                                     (257, 0, 72, 39424), (16, 9, 136, 58700), (32, 8, 72, 19456), (27, 18, 72, 13100),
+                                     (64, 9, 72, 600)])
+def test_lmhead_token_tiles_and_deal_exact_inputs(asd, B, K, H, V):
+    inp = inputs.gen_lmhead_exact(B, K, H, V, 7900 + B + K + H, "cuda")
+    T = B * (K + 1)
+    led = asd.make_ledger(B, 8.0)
+    out = asd.lmhead_verify(inp.hidden, inp.weight, inp.draft, led, 1.0, 2)
+    logits = asd.lmhead_logits(inp.hidden, inp.weight)
+    torch.cuda.synchronize()
+    z64 = oracle.lmhead_logits_matmul(inp.hidden.cpu(), inp.weight.cpu())
+    z32 = z64.astype(np.float32)
+    assert np.array_equal(z64, z32.astype(np.float64)), "integer inputs must give exact logits"
+    assert np.array_equal(logits.cpu().numpy(), z32)
+    o = oracle.verify(z32.reshape(B, K + 1, V), inp.draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), 1.0, 2)
+    for key in ("accepted_len", "committed", "recovery", "row_argmax", "status"):
+        assert np.array_equal(out[key].cpu().numpy(), o[key]), key
+    assert np.array_equal(out["row_top"].cpu().numpy().reshape(T), z32.max(axis=1))
+    assert np.array_equal(out["row_regret"].cpu().numpy().view(np.uint32), o["row_regret"].view(np.uint32))
+    assert np.array_equal(led.cpu().numpy().view(np.uint32), o["ledger"].view(np.uint32))
+
+
 @pytest.mark.parametrize("B,K,H,V", [(8, 8, 512, 1000), (40, 8, 256, 2100), (5, 0, 64, 777), (3, 16, 320, 1300),
                                      (1500, 9, 64, 300), (6, 8, 8, 1000), (7, 3, 40, 513)])
 def test_lmhead_verify_exact_inputs_bit_exact(asd, B, K, H, V):
