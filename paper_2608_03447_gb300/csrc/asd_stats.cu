@@ -39,7 +39,8 @@ __global__ void __launch_bounds__(kStatThreads)
   const int ncount = a.ntau * a.np;
   for (int i = threadIdx.x; i <= ncount; i += blockDim.x) local[i] = 0u;
   // programmatic dependent launch: the next kernel may start its set-up now;
-  // this one reads the verify outputs only once the kernel before it is done
+  // this one reads the verify outputs only once the kernel before it is done,
+  // and past L1, which an earlier call of this kernel may have filled meanwhile
   pdl_signal_dependents();
   pdl_wait_prerequisites();
   __syncthreads();
@@ -52,11 +53,11 @@ __global__ void __launch_bounds__(kStatThreads)
     int xj = 0, yj = 0;
     float rj = 0.0f;
     if (mine) {
-      xj = draft[b * K + lane];
-      yj = row_argmax[b * (K + 1) + lane];
-      rj = row_regret[b * K + lane];
+      xj = __ldcg(draft + b * K + lane);
+      yj = __ldcg(row_argmax + b * (K + 1) + lane);
+      rj = __ldcg(row_regret + b * K + lane);
     }
-    const int st = status ? status[b] : 0;
+    const int st = status ? __ldcg(status + b) : 0;
     if (st == 0) {
       const uint32_t m = __ballot_sync(kFullMask, mine && xj == yj);
       const uint32_t all = K >= 32 ? 0xffffffffu : ((1u << K) - 1u);
@@ -131,20 +132,30 @@ __global__ void __launch_bounds__(kCommitThreads) commit_kernel(int B, int K, co
                                                                 const int32_t* __restrict__ committed, int pending,
                                                                 int32_t* kv_len, int32_t* tokens, int32_t* token_len,
                                                                 int max_tokens, int32_t* status) {
+  // Programmatic dependent launch: the next call's kernels may become resident
+  // now, and this one touches nothing before the kernel ahead of it is done.
+  // The work is a few loads and stores, so the launch is what it costs; worse,
+  // a plain launch ended the chain, and a verify on resident inputs behind it
+  // could not stream while the step before finished: 28.8 -> 12.6 us per step of
+  // verify + opportunity + commit at B=32, K=8, V=151936 bf16 (12.0 verify
+  // alone). Loads go past L1: a line of it may be older than the kernel ahead.
+  pdl_signal_dependents();
+  pdl_wait_prerequisites();
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * (kCommitThreads / 32) + (threadIdx.x >> 5);
   if (b >= B) return;
-  int a = accepted_len[b];
+  int a = __ldcg(accepted_len + b);
   a = a < 0 ? 0 : (a > K ? K : a);  // asd_verify writes 0..K; anything else is clamped (memory safety)
-  const int len = tokens ? token_len[b] : 0;
+  const int len = tokens ? __ldcg(token_len + b) : 0;
   const bool room = !tokens || len + a + 1 <= max_tokens;
   if (tokens && room && lane <= a)
-    tokens[static_cast<long long>(b) * max_tokens + len + lane] = committed[static_cast<long long>(b) * (K + 1) + lane];
+    tokens[static_cast<long long>(b) * max_tokens + len + lane] =
+        __ldcg(committed + static_cast<long long>(b) * (K + 1) + lane);
   if (lane == 0) {
     if (status) status[b] = room ? 0 : ASD_STATUS_OVERFLOW;
     if (room) {
       if (tokens) token_len[b] = len + a + 1;
-      if (kv_len) kv_len[b] += pending + a;
+      if (kv_len) kv_len[b] = __ldcg(kv_len + b) + pending + a;
     }
   }
 }
@@ -158,11 +169,12 @@ extern "C" int asd_commit(int B, int K, const int32_t* accepted_len, const int32
   if (B == 0) return ASD_OK;
   if (!accepted_len || !committed) return ASD_ERR_NULL;
   if (tokens && (!token_len || max_tokens < 1)) return ASD_ERR_NULL;
-  // a plain launch: with programmatic dependent launch it measured slower
-  // behind a kernel that does not trigger its dependents early
   constexpr int kWarps = kCommitThreads / 32;
-  commit_kernel<<<static_cast<unsigned>((B + kWarps - 1) / kWarps), kCommitThreads, 0,
-                  reinterpret_cast<cudaStream_t>(stream)>>>(B, K, accepted_len, committed, pending, kv_len, tokens,
-                                                            token_len, max_tokens, status);
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = pdl_config(dim3(static_cast<unsigned>((B + kWarps - 1) / kWarps)),
+                                            dim3(kCommitThreads), reinterpret_cast<cudaStream_t>(stream), &attr);
+  if (cudaLaunchKernelEx(&cfg, commit_kernel, B, K, accepted_len, committed, pending, kv_len, tokens, token_len,
+                         max_tokens, status) != cudaSuccess)
+    return ASD_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
 }
