@@ -353,8 +353,8 @@ int asd_commit(int B, int K, const int32_t* accepted_len, const int32_t* committ
 int asd_host_alias(const void* host, void** device);
 
 /* How many kernels one asd_verify / asd_verify_strict call launches for this
- * shape (1 or 2: the row stage, and for large inputs a separate selection
- * kernel launched right behind it); 0 for B = 0. For accounting only. */
+ * shape (1 or 2: the row stage, and unless the row stage selects as well a
+ * selection kernel launched right behind it); 0 for B = 0. For accounting only. */
 int asd_verify_launches(int B, int K, int V, int dtype, int* launches);
 
 /* Launch options of the logit-streaming entry points (asd_verify,
@@ -362,13 +362,14 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches);
  * The paper has no counterpart: these choose among kernels that compute the
  * same results bit for bit, for tests that cover each kernel and for
  * measurements; the defaults (all fields 0) are what production calls want.
- *   path          ASD_PATH_AUTO picks the row-stage kernel by input size (the
+ *   path          ASD_PATH_AUTO picks the row-stage kernel by size (the
  *                 one-CTA-per-request kernel below 1 MB when a request fits
- *                 it, the register-streaming kernel for other small inputs,
- *                 the TMA pipeline from 1 MB); the others force one (a forced
+ *                 it, the TMA pipeline for ASD_RESIDENT_INPUTS of at least 1 MB
+ *                 in rows of at least 112 KB, the register-streaming kernel for
+ *                 everything else); the others force one (a forced
  *                 ASD_PATH_SMALL falls back to AUTO where the shape does not
  *                 fit it).
- *   fused_select  1: the TMA row stage runs the selection itself (the CTA that
+ *   fused_select  1: the row stage runs the selection itself (the CTA that
  *                 completes a request selects it) instead of launching
  *                 select_kernel right behind it.
  *   no_pdl        1: launch without programmatic dependent launch.

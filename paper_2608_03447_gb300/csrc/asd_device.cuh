@@ -19,7 +19,6 @@ struct VerifyParams {
   int B, K, V;
   long long total;     // B * (K+1) * V elements
   long long head;      // elements before the first 16-byte boundary
-  long long per_warp;  // elements per warp after the head (multiple of the vector width)
   const int32_t* draft;
   asd_ledger* ledger;
   float gate;
@@ -50,6 +49,7 @@ template <typename T> struct Elem;
 template <> struct Elem<float> {
   static constexpr int kVec = 4;  // elements per 128-bit vector
   static __device__ __forceinline__ float load(const float* p, long long i) { return __ldg(p + i); }
+  static __device__ __forceinline__ float load_cg(const float* p, long long i) { return __ldcg(p + i); }
   static __device__ __forceinline__ float lane(const uint4& v, int t) {
     const uint32_t w = t == 0 ? v.x : t == 1 ? v.y : t == 2 ? v.z : v.w;
     return __uint_as_float(w);
@@ -60,6 +60,10 @@ template <> struct Elem<__nv_bfloat16> {
   static __device__ __forceinline__ float load(const __nv_bfloat16* p, long long i) {
     const unsigned short bits = __ldg(reinterpret_cast<const unsigned short*>(p) + i);
     return __uint_as_float(static_cast<uint32_t>(bits) << 16);  // bf16 -> fp32 is exact
+  }
+  static __device__ __forceinline__ float load_cg(const __nv_bfloat16* p, long long i) {
+    const unsigned short bits = __ldcg(reinterpret_cast<const unsigned short*>(p) + i);
+    return __uint_as_float(static_cast<uint32_t>(bits) << 16);
   }
   static __device__ __forceinline__ float lane(const uint4& v, int t) {
     const int q = t >> 1;

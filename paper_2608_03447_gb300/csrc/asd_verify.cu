@@ -3,25 +3,23 @@
 // asd_verify_blocks, asd_shard_partials and asd_verify_noalloc.
 //
 // A step is two stages over the [B, K+1, V] logits, treated as one flat array:
-//   row stage  (Eq. 1, Eq. 3) the flat array is cut into equal, 16-byte
-//              aligned ranges; each range is streamed with 128-bit loads (or
+//   row stage  (Eq. 1, Eq. 3) pieces of rows are streamed with 128-bit loads (or
 //              TMA bulk copies into a shared-memory ring), every lane keeps a
 //              NaN-propagating running maximum, and each row segment reduces
 //              to one 64-bit key (order-preserving fp32 bits, then the
 //              inverted vocabulary index) merged into the row's slot by
 //              atomicMax: the largest key is the largest logit at the lowest
-//              index, whatever order the segments finish in. The segment that
-//              holds the draft token also records z_j(x_j).
+//              index, whatever order the segments finish in. z_j(x_j), the draft
+//              token's logit, is recorded beside it.
 //   selection  (Eq. 5-13, Alg. 1) one warp per request, lane j owning target
 //              row j, resets the request's workspace slots to zero as it reads
 //              them, so the workspace is zero again after every call (whatever
 //              shape the next call has).
-// Three row-stage kernels cover the input sizes: verify_small_kernel (one CTA
-// per request, selection in the same CTA) below 1 MB when a request fits one
-// round of loads, verify_kernel (register streaming; the warp that completes a
-// request selects it) for other small inputs, and verify_tma_kernel from 1 MB,
-// followed by select_kernel (or, as a launch option, selecting in the CTA that
-// completes each request).
+// Three row-stage kernels (choose_path): verify_small_kernel (one CTA per
+// request, selection in the same CTA) for small requests, verify_stream_kernel
+// (one piece of one row per warp) for most calls, and verify_tma_kernel for
+// long rows declared resident. The latter two are followed by select_kernel
+// (or, as a launch option, select in the CTA that completes each request).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -37,26 +35,19 @@ namespace {
 
 using namespace asd_detail;
 
-// Tuning constants (overridable at build time for launch-shape sweeps).
-#ifndef ASD_VERIFY_THREADS
-#define ASD_VERIFY_THREADS 256
-#endif
-#ifndef ASD_VERIFY_UNROLL
-#define ASD_VERIFY_UNROLL 4
-#endif
-#ifndef ASD_VERIFY_MIN_BLOCKS
-#define ASD_VERIFY_MIN_BLOCKS 0  // 0: no residency hint to the register allocator
-#endif
-#ifndef ASD_VERIFY_MIN_ELEMS_PER_WARP
-#define ASD_VERIFY_MIN_ELEMS_PER_WARP 2048
-#endif
-constexpr int kThreads = ASD_VERIFY_THREADS;
+constexpr int kThreads = 128;  // of verify_stream_kernel
 constexpr int kWarpsPerBlock = kThreads / 32;
-constexpr int kUnroll = ASD_VERIFY_UNROLL;  // 128-bit loads in flight per lane
-constexpr long long kMinElemsPerWarp = ASD_VERIFY_MIN_ELEMS_PER_WARP;
+// Vectors per lane of a unit, all in flight at once: eight (4 KB units), or four
+// where the input is spread thinner than that. Nine CTAs per SM keep the eight
+// in registers without spills.
+constexpr int kStreamUnroll = 8;
+constexpr int kStreamUnrollSmall = 4;
+constexpr int kStreamMinBlocks = 9;
+// A weak (coherent) load: with programmatic dependent launch this kernel may be
+// resident while an earlier one writes what it will read after the wait.
 __device__ __forceinline__ uint4 load_stream(const uint4* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
@@ -82,7 +73,7 @@ __device__ __forceinline__ float vec_max(const uint4& v, __nv_bfloat16) {
 
 // Reduces elements [s0, s1) of one row (which starts at flat index row0) to a
 // key; every lane returns the warp's key. Sets *nan when a NaN was seen.
-template <typename T, int kU = kUnroll>
+template <typename T, int kU>
 __device__ __forceinline__ unsigned long long segment_key(const T* z, long long s0, long long s1,
                                                           long long row0, long long head,
                                                           int lane, bool* nan) {
@@ -174,77 +165,223 @@ __device__ __forceinline__ unsigned long long segment_key(const T* z, long long 
   return warp_max_key(key);
 }
 
-// ---------------------------------------------------------------- the fused kernel
+// ---------------------------------------------------------------- register-streaming kernel
+//
+// One warp takes one unit: up to 256 vectors (4 KB) of ONE row, all of
+// its loads in flight at once, and exits. There is no loop, no ring and no row
+// change: which row, which part of it and where its vectors lie is arithmetic
+// done before the wait for the previous kernel; what follows the loads is a
+// register maximum, one warp reduction and the index search in the lanes that
+// hold the warp's maximum. Units are dealt by the hardware as CTAs retire, so no
+// CTA's share can end late. The first q.draft_ctas CTAs fetch the draft tokens'
+// logits instead, a row per thread.
+//
+// Bound by memory: a kernel that only loads the same bytes this way takes 13.3 us
+// for 87.5 MB and 88.5 us for 662 MB where a call, selection included, takes 15.5
+// and 93 us (the TMA pipeline: 20.5 and 100). What else was measured: 2 KB units
+// with twice the warps 16.0 / 93.2 us; every warp reducing to the row's slot by
+// itself 16.3 / 95.6 us (and 18.4 / 108 us with 2 KB units: the slots of
+// neighbouring rows share a line of L2, which takes them one by one); units that
+// do not end on 128-byte lines, 17.2 / 95.5 us.
+struct StreamPlan {
+  unsigned draft_ctas;  // CTAs that fetch draft logits
+  unsigned rows;
+  unsigned total;       // units in all
+  int units;            // units per row
+  int per;              // vectors per unit, a multiple of 32
+  int line;             // where in its 128-byte line the first vector of the logits lies
+  // n / d = (n * mul) >> shift for n < 2^31
+  struct Divide {
+    unsigned mul, shift;
+    void set(unsigned d) {
+      unsigned l = 0;
+      while ((1ull << l) < d) ++l;
+      mul = static_cast<unsigned>((1ull << (31 + l)) / d + 1);
+      shift = 31 + l;
+    }
+    __device__ __forceinline__ unsigned operator()(unsigned n) const {
+      return static_cast<unsigned>((static_cast<unsigned long long>(n) * mul) >> shift);
+    }
+  };
+  Divide by_units, by_k1;
+};
 
-#if ASD_VERIFY_MIN_BLOCKS > 0
-#define ASD_VERIFY_BOUNDS __launch_bounds__(kThreads, ASD_VERIFY_MIN_BLOCKS)
-#else
-#define ASD_VERIFY_BOUNDS __launch_bounds__(kThreads)
-#endif
+// The first element of v equal to m, its maximum; VN - 1 if none (m is NaN).
+template <typename T>
+__device__ __forceinline__ int vec_first_equal(const uint4& v, float m) {
+  int first = Elem<T>::kVec - 1;
+#pragma unroll
+  for (int t = Elem<T>::kVec - 1; t >= 0; --t)
+    if (Elem<T>::lane(v, t) == m) first = t;
+  return first;
+}
 
+// The packed maximum of several 128-bit vectors, kept packed until the end.
+__device__ __forceinline__ uint32_t packed_max(uint32_t a, uint32_t b, float) {
+  return __float_as_uint(fmax_nan(__uint_as_float(a), __uint_as_float(b)));
+}
+__device__ __forceinline__ uint32_t packed_max(uint32_t a, uint32_t b, __nv_bfloat16) {
+  uint32_t m;
+  asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(a), "r"(b));
+  return m;
+}
+__device__ __forceinline__ float packed_value(uint32_t m, float) { return __uint_as_float(m); }
+__device__ __forceinline__ float packed_value(uint32_t m, __nv_bfloat16) {
+  return fmax_nan(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
+}
+template <typename T>
+__device__ __forceinline__ uint32_t packed_max(const uint4& v) {
+  return packed_max(packed_max(v.x, v.y, T()), packed_max(v.z, v.w, T()), T());
+}
+
+__device__ __forceinline__ float warp_max_nan(float v) {
+  float m;
+  asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+  return m;
+}
+
+// VN u + t: element t of v[u] is the first that equals best, one of them does.
+template <typename T, int u, int kU>
+__device__ __forceinline__ int first_holding(const uint4 (&v)[kU], float best) {
+  if constexpr (u + 1 < kU) {
+    if (packed_value(packed_max<T>(v[u]), T()) != best) return first_holding<T, u + 1>(v, best);
+  }
+  return Elem<T>::kVec * u + vec_first_equal<T>(v[u], best);
+}
+
+// Adds n to its request's counter and runs the selections that this completes
+// (each lane with its own request; lanes with n = 0 add nothing).
 template <typename T, bool kStrict>
-__global__ void ASD_VERIFY_BOUNDS verify_kernel(const VerifyParams p) {
+__device__ __noinline__ void count_and_select(const VerifyParams& p, unsigned request, unsigned n, int lane) {
+  bool complete = false;
+  if (n > 0) {
+    __threadfence();
+    const unsigned long long old = atomicAdd(&p.done[request], static_cast<unsigned long long>(n));
+    // every element, and every row once for its draft logit
+    complete = old + n == static_cast<unsigned long long>(p.K + 1) * (static_cast<unsigned long long>(p.V) + 1) * p.nblk;
+  }
+  for (unsigned left = __ballot_sync(kFull, complete); left; left &= left - 1) {
+    __threadfence();
+    select_request<T, kStrict>(p, static_cast<int>(__shfl_sync(kFull, request, __ffs(left) - 1)), lane);
+  }
+}
+
+template <typename T, bool kStrict, bool kSplit, int kU>
+__global__ void __launch_bounds__(kThreads, kSplit ? kStreamMinBlocks : 1)
+    verify_stream_kernel(const __grid_constant__ VerifyParams p, const __grid_constant__ StreamPlan q) {
+  constexpr int VN = Elem<T>::kVec;
   const int lane = threadIdx.x & 31;
-  const long long warp = static_cast<long long>(blockIdx.x) * kWarpsPerBlock + (threadIdx.x >> 5);
-  const long long lo = warp == 0 ? 0 : p.head + warp * p.per_warp;
-  long long hi = p.head + (warp + 1) * p.per_warp;
-  hi = hi < p.total ? hi : p.total;
-  if (lo >= hi) return;
-
-  const T* z = static_cast<const T*>(p.logits);
-  const int V = p.V, K = p.K, K1 = p.K + 1;
-  // counters are per request; a request is complete when all p.nblk of its blocks are
-  const unsigned long long request_elems = static_cast<unsigned long long>(K1) * V * p.nblk;
-
-  long long row = lo / V;
-  int pending_b = static_cast<int>(row / K1);
-  unsigned long long pending_n = 0;
-
-  for (long long s0 = lo; s0 < hi; ++row) {
-    const long long row0 = row * V;
-    const long long s1 = hi < row0 + V ? hi : row0 + V;
-    const int b = static_cast<int>(row / K1);
-    const int j = static_cast<int>(row - static_cast<long long>(b) * K1);
-    int x = -1;
-    if (j < K) x = __ldg(p.draft + static_cast<long long>(b) * K + j) - p.v_offset;  // shard-local
-
-    if (b != pending_b) {  // finished this warp's share of block-request pending_b
-      bool last = false;
-      if (lane == 0) {
-        __threadfence();
-        const unsigned long long old = atomicAdd(&p.done[pending_b % p.B], pending_n);
-        last = old + pending_n == request_elems;
-      }
-      if (__shfl_sync(kFull, last, 0)) {
-        __threadfence();
-        select_request<T, kStrict>(p, pending_b % p.B, lane);
-      }
-      pending_b = b;
-      pending_n = 0;
+  const int V = p.V;
+  pdl_signal_dependents();
+  if (blockIdx.x < q.draft_ctas) {
+    const unsigned row = blockIdx.x * kThreads + threadIdx.x;
+    const unsigned b = q.by_k1(row);
+    if (!p.resident) pdl_wait_prerequisites();
+    float zx = 0.0f;
+    bool has_zx = false;
+    if (row < q.rows && row - b * (p.K + 1) < static_cast<unsigned>(p.K)) {
+      const int x = __ldcg(p.draft + (row - b)) - p.v_offset;  // row = b (K + 1) + j, its draft at b K + j; shard-local
+      has_zx = x >= 0 && x < V;
+      if (has_zx) zx = Elem<T>::load_cg(static_cast<const T*>(p.logits), static_cast<long long>(row) * V + x);
     }
-
-    bool nan = false;
-    const unsigned long long key = segment_key<T>(z, s0, s1, row0, p.head, lane, &nan);
-    if (lane == 0) {
-      atomicMax(&p.row_key[row], key);
-      if (nan) atomicOr(&p.flags[b], ASD_STATUS_NAN_LOGIT);
-      if (x >= 0 && x < V && row0 + x >= s0 && row0 + x < s1)
-        p.draft_logit[row] = Elem<T>::load(z, row0 + x);
-    }
-    pending_n += static_cast<unsigned long long>(s1 - s0);
-    s0 = s1;
+    pdl_wait_prerequisites();  // resident inputs: before the first touch of the workspace
+    if (has_zx) p.draft_logit[row] = zx;
+    if (!kSplit) count_and_select<T, kStrict>(p, b % static_cast<unsigned>(p.B), row < q.rows ? 1u : 0u, lane);
+    return;
   }
+  __shared__ unsigned long long s_key[kWarpsPerBlock];
+  __shared__ unsigned s_row[kWarpsPerBlock], s_count[kWarpsPerBlock];
+  const int warp = threadIdx.x >> 5;
+  const unsigned unit = (blockIdx.x - q.draft_ctas) * kWarpsPerBlock + warp;
+  const unsigned row = q.by_units(unit);
+  const int k = static_cast<int>(unit - row * q.units);
+  // The row's elements: loose ones up to the first 16-byte boundary, nvec whole
+  // vectors, loose ones again. Units meet on 128-byte lines, so that a line is
+  // read by one load of one warp.
+  const long long row0 = static_cast<long long>(row) * V;
+  const long long past = row0 - p.head;
+  int lead = static_cast<int>(past <= 0 ? -past : -past & (VN - 1));
+  lead = lead < V ? lead : V;
+  const int nvec = (V - lead) / VN;
+  const int line = static_cast<int>((past + lead) / VN + q.line) & 7;
+  const bool first = k == 0, last = k == q.units - 1;
+  const int v0 = first ? 0 : min(k * q.per - line, nvec);
+  const int v1 = last ? nvec : min((k + 1) * q.per - line, nvec);
+  const T* z = static_cast<const T*>(p.logits) + row0;
 
-  bool last = false;
+  // The logits may be the previous kernel's unless the caller declared them
+  // resident; the workspace is touched after the wait below.
+  if (!p.resident) pdl_wait_prerequisites();
+  const bool mine_exists = unit < q.total;
+  const int n = v1 - v0;
+  unsigned long long key = 0ull;
+  if (mine_exists && n > 0) {
+    // past its end a unit repeats its last vector, which changes no maximum and no index
+    const uint4* vp = reinterpret_cast<const uint4*>(z + lead) + v0;
+    uint4 v[kU];
+    if (n == 32 * kU) {
+#pragma unroll
+      for (int u = 0; u < kU; ++u) v[u] = load_stream(vp + lane + 32 * u);
+    } else {
+#pragma unroll
+      for (int u = 0; u < kU; ++u) v[u] = load_stream(vp + min(lane + 32 * u, n - 1));
+    }
+    uint32_t packed = packed_max<T>(v[0]);
+#pragma unroll
+    for (int u = 1; u < kU; ++u) packed = packed_max(packed, packed_max<T>(v[u]), T());
+    const float mine = packed_value(packed, T());
+    const float best = warp_max_nan(mine);
+    unsigned at = 0xffffffffu;  // the lowest index that holds it; with a NaN in the unit none does
+    if (mine == best) {
+      const int first_at = first_holding<T, 0>(v, best);
+      at = lead + (v0 + min(lane + 32 * (first_at / VN), n - 1)) * VN + first_at % VN;
+    }
+    at = __reduce_min_sync(kFull, at);
+    if (best == best) {
+      key = make_key(best, at);
+    } else if (lane == 0) {
+      pdl_wait_prerequisites();
+      atomicOr(&p.flags[q.by_k1(row)], ASD_STATUS_NAN_LOGIT);
+    }
+  }
+  if (mine_exists && ((first && lead > 0) || (last && lead + nvec * VN < V))) {
+    // loose elements, fewer than VN on either side: one per lane, each merged by itself
+    pdl_wait_prerequisites();
+    const int e = lane < VN ? lane : lead + nvec * VN + lane - VN;
+    if (lane < VN ? first && e < lead : last && lane < 2 * VN && e < V) {
+      const float loose = Elem<T>::load_cg(z, e);
+      if (loose == loose) {
+        atomicMax(&p.row_key[row], make_key(loose, static_cast<uint32_t>(e)));
+      } else {
+        atomicOr(&p.flags[q.by_k1(row)], ASD_STATUS_NAN_LOGIT);
+      }
+    }
+  }
+  // one reduction per row and CTA
   if (lane == 0) {
-    __threadfence();
-    const unsigned long long old = atomicAdd(&p.done[pending_b % p.B], pending_n);
-    last = old + pending_n == request_elems;
+    s_key[warp] = key;
+    s_row[warp] = mine_exists ? row : 0xffffffffu;
+    if (!kSplit) {
+      const int rel0 = first ? 0 : lead + v0 * VN, rel1 = last ? V : lead + v1 * VN;
+      s_count[warp] = mine_exists ? static_cast<unsigned>(rel1 - rel0) : 0u;
+    }
   }
-  if (__shfl_sync(kFull, last, 0)) {
-    __threadfence();
-    select_request<T, kStrict>(p, pending_b % p.B, lane);
+  if (!kSplit) __threadfence();
+  pdl_wait_prerequisites();  // resident inputs: before the first touch of the workspace
+  __syncthreads();
+  if (warp != 0) return;
+  const unsigned r = lane < kWarpsPerBlock ? s_row[lane] : 0xffffffffu;
+  unsigned long long m = lane < kWarpsPerBlock ? s_key[lane] : 0ull;
+#pragma unroll
+  for (int d = 1; d < kWarpsPerBlock; d *= 2) {
+    const unsigned long long o = __shfl_down_sync(kFull, m, d);
+    if (__shfl_down_sync(kFull, r, d) == r && o > m) m = o;
   }
+  const unsigned before = __shfl_up_sync(kFull, r, 1);
+  if (m != 0ull && (lane == 0 || before != r)) atomicMax(&p.row_key[r], m);
+  if (!kSplit)  // the warp that completes a request (all p.nblk of its blocks) selects it
+    count_and_select<T, kStrict>(p, q.by_k1(r) % static_cast<unsigned>(p.B),
+                                 lane < kWarpsPerBlock ? s_count[lane] : 0u, lane);
 }
 
 // ---------------------------------------------------------------- one CTA per request (small inputs)
@@ -438,16 +575,6 @@ __device__ __forceinline__ float smem_elem(const uint4* src, int off, __nv_bfloa
   unsigned short bits;
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(bits) : "r"(smem_u32(src) + 2u * static_cast<uint32_t>(off)));
   return __uint_as_float(static_cast<uint32_t>(bits) << 16);
-}
-
-// The first element of v equal to m, its maximum; VN - 1 if none (m is NaN).
-template <typename T>
-__device__ __forceinline__ int vec_first_equal(const uint4& v, float m) {
-  int first = Elem<T>::kVec - 1;
-#pragma unroll
-  for (int t = Elem<T>::kVec - 1; t >= 0; --t)
-    if (Elem<T>::lane(v, t) == m) first = t;
-  return first;
 }
 
 // Merges one warp's partial result for a row into the workspace: the row's
@@ -784,6 +911,7 @@ __global__ void __launch_bounds__(kTmaThreads, ASD_TMA_MIN_BLOCKS)
         }
       }
     }
+    pdl_wait_prerequisites();  // this grid completes after the one before it, whatever happened here
     return;
   }
   // The first touch of the workspace: wait for the previous launch, flush the
@@ -819,36 +947,6 @@ __global__ void __launch_bounds__(kTmaThreads, ASD_TMA_MIN_BLOCKS)
 }
 
 // ---------------------------------------------------------------- host side
-
-// Resident warps of a kernel on the current device, queried once per device.
-template <typename T, bool kStrict>
-int resident_warps(int* out) {
-  constexpr int kMaxDevices = 64;
-  static int cache[kMaxDevices] = {0};
-  static std::mutex mu;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return ASD_ERR_CUDA;
-  if (dev >= 0 && dev < kMaxDevices) {
-    std::lock_guard<std::mutex> g(mu);
-    if (cache[dev] > 0) {
-      *out = cache[dev];
-      return ASD_OK;
-    }
-  }
-  int sms = 0, blocks = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return ASD_ERR_CUDA;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, verify_kernel<T, kStrict>, kThreads, 0) !=
-      cudaSuccess)
-    return ASD_ERR_CUDA;
-  const int w = sms * (blocks > 0 ? blocks : 1) * kWarpsPerBlock;
-  if (dev >= 0 && dev < kMaxDevices) {
-    std::lock_guard<std::mutex> g(mu);
-    cache[dev] = w;
-  }
-  *out = w;
-  return ASD_OK;
-}
 
 struct DeviceInfo {
   int sms = 0;
@@ -933,7 +1031,6 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
   if (per_cta < VN) per_cta = VN;
   ncta = bulk > 0 ? (bulk + per_cta - 1) / per_cta : 1;
   p.head = head;
-  p.per_warp = 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(ncta));
   cfg.blockDim = dim3(kTmaThreads);
@@ -957,24 +1054,85 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
   return launch_select<T, kStrict>(p, opt.pdl, stream);
 }
 
-// Which kernel streams the logits: the TMA pipeline for inputs of at least
-// kTmaMinBytes; below that, one CTA per request when a request fits one round
-// of loads of a CTA (single blocks, no vocabulary shard), else the
-// register-streaming kernel (fewer, shorter warps start faster on small
-// inputs). The launch options can force a kernel (the tests use that to cover
-// every kernel); a forced `small` falls back to the default when the shape does
-// not qualify.
+// Which kernel streams the logits.
+//   kTma     resident inputs of at least kTmaMinBytes whose rows are at least
+//            kTmaMinRowBytes: a slice is streamed ahead of the kernels before
+//            it, which a unit's CTA, that has to wait for them when it ends,
+//            cannot (12.0 against 15.8 us per step of 87.5 MB with 304 KB rows).
+//            A slice pays for every row it enters: at 200 MB the two meet
+//            between 100 KB rows (35.6 against 31.7 us) and 128 KB rows (30.0
+//            against 31.1 us).
+//   kSmall   one CTA per request, below kTmaMinBytes, when a request fits one
+//            round of loads of a CTA (single blocks, no vocabulary shard).
+//   kStream  everything else. A call that waits for the kernel ahead of it has
+//            nothing to overlap and takes 15.5 us for 87.5 MB where the TMA
+//            pipeline took 20.5 us, 93 against 100 us for 662 MB, 4.0 against
+//            8.2 us for 2.7 MB, 7.4 against 26 us for 16 MB in 2 KB rows.
+// The launch options can force a kernel (the tests use that to cover every
+// kernel); a forced `small` falls back to the default when the shape does not
+// qualify.
 constexpr long long kTmaMinBytes = 1LL << 20;
+constexpr long long kTmaMinRowBytes = 112LL << 10;
 
 enum class Path { kSmall, kStream, kTma };
 
-Path choose_path(int forced, long long bytes, long long request_bytes, int K, bool single_block) {
+Path choose_path(int forced, long long bytes, long long request_bytes, int K, bool single_block, bool resident) {
   const bool small_ok = single_block && K + 1 <= 32 && request_bytes <= kSmallMaxRequestBytes;
   if (forced == ASD_PATH_TMA) return Path::kTma;
   if (forced == ASD_PATH_STREAM) return Path::kStream;
   if (forced == ASD_PATH_SMALL && small_ok) return Path::kSmall;
-  if (bytes >= kTmaMinBytes) return Path::kTma;
-  return small_ok ? Path::kSmall : Path::kStream;
+  if (bytes < kTmaMinBytes) return small_ok ? Path::kSmall : Path::kStream;
+  return resident && request_bytes / (K + 1) >= kTmaMinRowBytes ? Path::kTma : Path::kStream;
+}
+
+// The cut of a row into units: as large as a warp's loads in flight allow, but
+// no larger than spreads a small input over kStreamWarpsPerSm warps on every SM.
+constexpr int kStreamWarpsPerSm = 16;
+constexpr long long kStreamMaxUnits = 1LL << 31;  // unit numbers are 32-bit
+
+template <typename T>
+StreamPlan stream_plan(const VerifyParams& p, long long rows, int sms) {
+  StreamPlan q = {};
+  const long long nvec = p.V / Elem<T>::kVec;  // whole vectors of a row, at most
+  const long long warps = static_cast<long long>(sms) * kStreamWarpsPerSm;
+  long long per = ((rows * nvec + warps - 1) / warps + 31) / 32 * 32;
+  per = per < 32 ? 32 : per > 32 * kStreamUnroll ? 32 * kStreamUnroll : per;
+  q.per = static_cast<int>(per);
+  q.units = nvec <= per ? 1 : static_cast<int>((nvec + 7 + per - 1) / per);  // + 7: the first unit may begin inside a line
+  q.line = static_cast<int>((reinterpret_cast<uintptr_t>(p.logits) + static_cast<size_t>(p.head) * sizeof(T)) / 16 % 8);
+  q.rows = static_cast<unsigned>(rows);
+  q.by_units.set(static_cast<unsigned>(q.units));
+  q.by_k1.set(static_cast<unsigned>(p.K + 1));
+  return q;
+}
+
+template <typename T, bool kStrict, bool kSplit>
+int launch_stream(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
+  int dev = 0;
+  DeviceInfo* info = nullptr;
+  const int rc = device_info(&dev, &info);
+  if (rc != ASD_OK) return rc;
+  const long long rows = static_cast<long long>(p.nblk) * p.B * (p.K + 1);
+  StreamPlan q = stream_plan<T>(p, rows, info->sms);
+  if (rows >= kStreamMaxUnits / q.units) return launch_tma<T, kStrict>(p, opt, stream);
+  q.total = static_cast<unsigned>(rows * q.units);
+  q.draft_ctas = p.K > 0 || !kSplit ? static_cast<unsigned>((rows + kThreads - 1) / kThreads) : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(q.draft_ctas + static_cast<unsigned>((rows * q.units + kWarpsPerBlock - 1) / kWarpsPerBlock));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  if (opt.pdl) {
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  auto kernel = q.per <= 32 * kStreamUnrollSmall ? verify_stream_kernel<T, kStrict, kSplit, kStreamUnrollSmall>
+                                                 : verify_stream_kernel<T, kStrict, kSplit, kStreamUnroll>;
+  if (cudaLaunchKernelEx(&cfg, kernel, p, q) != cudaSuccess) return ASD_ERR_CUDA;
+  if (kSplit) return launch_select<T, kStrict>(p, opt.pdl, stream);
+  return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
 }
 
 template <typename T, bool kStrict>
@@ -982,17 +1140,15 @@ int launch(VerifyParams& p, cudaStream_t stream) {
   const long long request_bytes = static_cast<long long>(p.K + 1) * p.V * static_cast<long long>(sizeof(T));
   const LaunchOptions opt = launch_options();
   const Path path = choose_path(opt.path, p.total * static_cast<long long>(sizeof(T)), request_bytes, p.K,
-                                p.nblk == 1 && !p.partials);
+                                p.nblk == 1 && !p.partials, p.resident != 0);
   if (path == Path::kTma) return launch_tma<T, kStrict>(p, opt, stream);
-  constexpr int VN = Elem<T>::kVec;
   const uintptr_t addr = reinterpret_cast<uintptr_t>(p.logits);
   if (addr % sizeof(T) != 0) return ASD_ERR_ALIGN;
   long long head = static_cast<long long>(((16 - addr % 16) % 16) / sizeof(T));
   if (head > p.total) head = p.total;
   if (path == Path::kSmall) {
     p.head = head;
-    p.per_warp = 0;
-    cudaLaunchConfig_t cfg = {};
+      cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(p.B));
     cfg.blockDim = dim3(kSmallThreads);
     cfg.stream = stream;
@@ -1006,23 +1162,8 @@ int launch(VerifyParams& p, cudaStream_t stream) {
     if (cudaLaunchKernelEx(&cfg, verify_small_kernel<T, kStrict>, p) != cudaSuccess) return ASD_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
   }
-  const long long rest = p.total - head;
-  int max_warps = 0;
-  const int rc = resident_warps<T, kStrict>(&max_warps);
-  if (rc != ASD_OK) return rc;
-  long long nw = (rest + kMinElemsPerWarp - 1) / kMinElemsPerWarp;
-  if (nw > max_warps) nw = max_warps;
-  if (nw < 1) nw = 1;
-  long long per_warp = (rest + nw - 1) / nw;
-  per_warp = (per_warp + VN - 1) / VN * VN;
-  if (per_warp < VN) per_warp = VN;
-  nw = (rest + per_warp - 1) / per_warp;
-  if (nw < 1) nw = 1;
   p.head = head;
-  p.per_warp = per_warp;
-  const long long blocks = (nw + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  verify_kernel<T, kStrict><<<static_cast<unsigned>(blocks), kThreads, 0, stream>>>(p);
-  return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+  return opt.split ? launch_stream<T, kStrict, true>(p, opt, stream) : launch_stream<T, kStrict, false>(p, opt, stream);
 }
 
 int verify_common(bool strict, const void* logits, int dtype, int B, int K, int V,
@@ -1060,7 +1201,6 @@ int verify_common(bool strict, const void* logits, int dtype, int B, int K, int 
   p.partials = partials;
   p.total = static_cast<long long>(nblk) * B * (K + 1) * V;
   p.head = 0;
-  p.per_warp = 0;
   p.draft = draft;
   p.ledger = ledger;
   p.gate = gate;
@@ -1149,8 +1289,8 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches) {
   if (rc != ASD_OK) return rc;
   const long long request_bytes = static_cast<long long>(K + 1) * V * (dtype_code(dtype) == ASD_BF16 ? 2 : 4);
   const LaunchOptions opt = launch_options();
-  const Path path = choose_path(opt.path, request_bytes * B, request_bytes, K, true);
-  *launches = B == 0 ? 0 : (path == Path::kTma && opt.split ? 2 : 1);
+  const Path path = choose_path(opt.path, request_bytes * B, request_bytes, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0);
+  *launches = B == 0 ? 0 : (path != Path::kSmall && opt.split ? 2 : 1);
   return ASD_OK;
 }
 

@@ -1,0 +1,78 @@
+"""The register-streaming row stage at the sizes where its cut of a row into units can go wrong: one vector
+either side of a unit, a unit of one, four and eight loads per lane, rows shorter than a vector, starts off the
+16-byte and the 128-byte grid, rows whose maximum sits at a unit's edge or is tied across units, rows of -inf,
+infinities and the lowest finite value. Every output bit for bit the oracle's (comparisons and one fp32
+subtraction decide all of them)."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle
+
+pytestmark = pytest.mark.gpu
+
+VEC = {torch.bfloat16: 8, torch.float32: 4}
+
+
+def _equal(got, want, what):
+    for k in ("status", "accepted_len", "recovery", "committed", "row_argmax"):
+        assert np.array_equal(got[k].cpu().numpy(), want[k]), f"{what}: {k}"
+    g, o = got["row_regret"].cpu().numpy(), want["row_regret"]
+    assert ((g.view(np.uint32) == o.view(np.uint32)) | (np.isnan(g) & np.isnan(o))).all(), f"{what}: row_regret"
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("vectors", [0, 1, 31, 32, 33, 127, 128, 129, 255, 256, 257, 511, 513, 2049])
+def test_unit_edges(asd, dtype, vectors, fused):
+    vn = VEC[dtype]
+    rng = np.random.default_rng(vectors)
+    for extra, rows_mb in ((0, 0), (1, 0), (vn - 1, 12)):  # 12 MB of rows: eight loads per lane
+        V = vectors * vn + extra
+        if V < 1:
+            continue
+        K = 3
+        B = max(2, (rows_mb << 20) // ((K + 1) * V * (16 // vn)))
+        if B * (K + 1) > 6000:
+            continue  # the longer rows cover this
+        off = int(rng.integers(0, 64))
+        flat = torch.randn(off + B * (K + 1) * V, device="cuda").mul_(3.0).to(dtype)
+        z = flat[off:].view(B, K + 1, V)
+        tops = [0, V - 1, min(V - 1, 32 * vn), min(V - 1, 256 * vn - 1), min(V - 1, 256 * vn)]
+        for i, at in enumerate(tops[: K + 1]):
+            z[0, i, at] = 40.0
+        z[1, 0] = -math.inf                                  # no finite value: index 0
+        z[1, 1, [V - 1, V // 2]] = 50.0                      # a tie: the lower index
+        z[1, 2, V // 3] = math.inf
+        z[1, 3] = torch.finfo(dtype).min
+        draft = torch.randint(0, V, (B, K), dtype=torch.int32, device="cuda")
+        draft[:, 0] = z[:, 0].argmax(1)                      # the tops among the drafts, so longer prefixes occur
+        ledger = asd.make_ledger(B, 8.0)
+        try:
+            asd.set_launch_options(path="stream", fused_select=fused)
+            out = asd.verify(z, draft, ledger, 1.0, 2)
+            torch.cuda.synchronize()
+        finally:
+            asd.reset_launch_options()
+        want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), 1.0, 2)
+        _equal(out, want, f"V={V} off={off} {dtype}")
+        assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
+
+
+@pytest.mark.parametrize("row_bytes", [112 * 1024 - 2, 112 * 1024])
+@pytest.mark.parametrize("resident", [False, True])
+def test_both_sides_of_the_dispatch(asd, row_bytes, resident):
+    """Rows on both sides of the line between the two kernels for resident inputs, and of the 1 MB line."""
+    V, K = row_bytes // 2, 2
+    for B in (3, 4):
+        z = torch.randn(B, K + 1, V, device="cuda").mul_(3.0).to(torch.bfloat16)
+        draft = z[:, :K].argmax(2).to(torch.int32).contiguous()
+        draft[:, 1] = torch.randint(0, V, (B,), dtype=torch.int32, device="cuda")
+        ledger = asd.make_ledger(B, 8.0)
+        torch.cuda.synchronize()
+        out = asd.verify(z, draft, ledger, math.inf, 2, resident=resident)
+        torch.cuda.synchronize()
+        want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), math.inf, 2)
+        _equal(out, want, f"V={V} B={B}")
