@@ -140,7 +140,7 @@ __device__ __forceinline__ BlockInputs load_block(const VerifyParams& p, long lo
     p.row_key[row] = 0ull;  // the whole workspace is zero again after every call
   }
   if (lane < K) {
-    in.x = p.draft[vb * K + lane];
+    in.x = __ldcg(p.draft + vb * K + lane);
     in.zx = __ldcg(&p.draft_logit[row]);
     p.draft_logit[row] = 0.0f;
   }
@@ -282,8 +282,8 @@ __device__ void select_request(const VerifyParams& p, int b, int lane) {
   }
   float budget = 0.0f, spent = 0.0f;
   if (!kStrict && lane == 0) {
-    budget = p.ledger[b].budget;
-    spent = p.ledger[b].spent;
+    budget = __ldcg(&p.ledger[b].budget);
+    spent = __ldcg(&p.ledger[b].spent);
   }
   budget = __shfl_sync(kFull, budget, 0);
   spent = __shfl_sync(kFull, spent, 0);
