@@ -362,10 +362,11 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches);
  * The paper has no counterpart: these choose among kernels that compute the
  * same results bit for bit, for tests that cover each kernel and for
  * measurements; the defaults (all fields 0) are what production calls want.
- *   path          ASD_PATH_AUTO picks the row-stage kernel by size (the
- *                 one-CTA-per-request kernel below 1 MB when a request fits
- *                 it, the TMA pipeline for ASD_RESIDENT_INPUTS of at least 1 MB
- *                 in rows of at least 112 KB, the register-streaming kernel for
+ *   path          ASD_PATH_AUTO picks the row-stage kernel by size (one CTA or
+ *                 one cluster of CTAs per request, selection included, for few
+ *                 requests that fit it; the TMA pipeline for
+ *                 ASD_RESIDENT_INPUTS of at least 1 MB in rows of at least
+ *                 112 KB; the register-streaming kernel for
  *                 everything else); the others force one (a forced
  *                 ASD_PATH_SMALL falls back to AUTO where the shape does not
  *                 fit it).

@@ -15,8 +15,8 @@
 //              row j, resets the request's workspace slots to zero as it reads
 //              them, so the workspace is zero again after every call (whatever
 //              shape the next call has).
-// Three row-stage kernels (choose_path): verify_small_kernel (one CTA per
-// request, selection in the same CTA) for small requests, verify_stream_kernel
+// Three row-stage kernels (choose_path): verify_small_kernel (one CTA or cluster
+// per request, which selects it too) for few small requests, verify_stream_kernel
 // (one piece of one row per warp) for most calls, and verify_tma_kernel for
 // long rows declared resident. The latter two are followed by select_kernel
 // (or, as a launch option, select in the CTA that completes each request).
@@ -67,102 +67,6 @@ __device__ __forceinline__ float vec_max(const uint4& v, __nv_bfloat16) {
       : "=r"(m)
       : "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
   return fmax_nan(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
-}
-
-// ---------------------------------------------------------------- stage 1: one row segment
-
-// Reduces elements [s0, s1) of one row (which starts at flat index row0) to a
-// key; every lane returns the warp's key. Sets *nan when a NaN was seen.
-template <typename T, int kU>
-__device__ __forceinline__ unsigned long long segment_key(const T* z, long long s0, long long s1,
-                                                          long long row0, long long head,
-                                                          int lane, bool* nan) {
-  constexpr int VN = Elem<T>::kVec;
-  // the vector grid starts at `head`, the first 16-byte aligned element
-  const long long rel0 = s0 - head, rel1 = s1 - head;
-  long long bs = rel0 <= 0 ? head : head + ((rel0 + VN - 1) / VN) * VN;
-  bs = bs < s1 ? bs : s1;
-  long long be = rel1 <= 0 ? head : head + (rel1 / VN) * VN;
-  be = be < bs ? bs : (be > s1 ? s1 : be);
-
-  float best = -INFINITY;
-  long long best_i = -1;
-  bool saw_nan = false;
-
-  // body: whole vectors, lane l takes vectors l, l+32, ... in increasing order,
-  // so a strictly greater test keeps each lane's first occurrence
-  const long long nvec = (be - bs) / VN;
-  if (nvec > 0) {
-    const uint4* vp = reinterpret_cast<const uint4*>(z + bs);
-    float vbest = -INFINITY;
-    int bvec = -1;
-    uint4 saved = make_uint4(0, 0, 0, 0);
-    long long k = lane;
-    for (; k + 32 * (kU - 1) < nvec; k += 32 * kU) {
-      uint4 v[kU];
-#pragma unroll
-      for (int u = 0; u < kU; ++u) v[u] = load_stream(vp + k + 32 * u);
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const float m = vec_max(v[u], T());
-        const bool gt = m > vbest;
-        vbest = fmax_nan(vbest, m);
-        if (gt) {
-          saved = v[u];
-          bvec = static_cast<int>(k + 32 * u);
-        }
-      }
-    }
-    for (; k < nvec; k += 32) {
-      const uint4 v = load_stream(vp + k);
-      const float m = vec_max(v, T());
-      const bool gt = m > vbest;
-      vbest = fmax_nan(vbest, m);
-      if (gt) {
-        saved = v;
-        bvec = static_cast<int>(k);
-      }
-    }
-    if (vbest != vbest) saw_nan = true;
-    if (lane < nvec) {
-      if (bvec >= 0) {
-        int t_first = VN - 1;
-#pragma unroll
-        for (int t = VN - 1; t >= 0; --t)
-          if (Elem<T>::lane(saved, t) == vbest) t_first = t;
-        best = vbest;
-        best_i = bs + static_cast<long long>(bvec) * VN + t_first;
-      } else {
-        // every value this lane saw is -inf (or NaN, flagged): its first element stands
-        best = -INFINITY;
-        best_i = bs + static_cast<long long>(lane) * VN;
-      }
-    }
-  }
-
-  // ragged ends: fewer than one vector on each side, one element per lane
-  const long long n_head = bs - s0, n_tail = s1 - be;
-  if (lane < n_head || lane < n_tail) {
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const long long e = side == 0 ? s0 + lane : be + lane;
-      if (e >= (side == 0 ? bs : s1)) continue;
-      const float v = Elem<T>::load(z, e);
-      if (v != v) {
-        saw_nan = true;
-        continue;
-      }
-      if (best_i < 0 || v > best || (v == best && e < best_i)) {
-        best = v;
-        best_i = e;
-      }
-    }
-  }
-
-  *nan = __any_sync(kFull, saw_nan);
-  const unsigned long long key =
-      best_i < 0 ? 0ull : make_key(best, static_cast<uint32_t>(best_i - row0));
-  return warp_max_key(key);
 }
 
 // ---------------------------------------------------------------- register-streaming kernel
@@ -249,6 +153,77 @@ __device__ __forceinline__ int first_holding(const uint4 (&v)[kU], float best) {
   return Elem<T>::kVec * u + vec_first_equal<T>(v[u], best);
 }
 
+// A unit: part k of `units` of a row, cut every `per` vectors (a multiple of
+// 32). The row's elements are loose ones up to the first 16-byte boundary, nvec
+// whole vectors, loose ones again; the unit holds vectors [v0, v1), and the
+// row's first and last unit the loose elements. Units meet on 128-byte lines
+// (`line`: where in its line the logits' first vector lies), so that a line is
+// read by one load of one warp.
+template <typename T>
+struct Unit {
+  static constexpr int VN = Elem<T>::kVec;
+  const T* z;  // the row
+  int lead, nvec, v0, v1;
+  bool first, last;
+
+  __device__ __forceinline__ Unit(const VerifyParams& p, long long row, int k, int units, int per, int line) {
+    const int V = p.V;
+    const long long row0 = row * V;
+    const long long past = row0 - p.head;
+    lead = static_cast<int>(past <= 0 ? -past : -past & (VN - 1));
+    lead = lead < V ? lead : V;
+    nvec = (V - lead) / VN;
+    const int off = static_cast<int>((past + lead) / VN + line) & 7;
+    first = k == 0;
+    last = k == units - 1;
+    v0 = first ? 0 : min(k * per - off, nvec);
+    v1 = last ? nvec : min((k + 1) * per - off, nvec);
+    z = static_cast<const T*>(p.logits) + row0;
+  }
+  __device__ __forceinline__ int elements(int V) const {
+    return (last ? V : lead + v1 * VN) - (first ? 0 : lead + v0 * VN);
+  }
+  // The key of the vectors, at most 32 kU (every lane has it); 0 without any, or with a NaN among them.
+  template <int kU>
+  __device__ __forceinline__ unsigned long long vectors(int lane, bool& nan) const {
+    const int n = v1 - v0;
+    if (n <= 0) return 0ull;
+    // past its end a unit repeats its last vector, which changes no maximum and no index
+    const uint4* vp = reinterpret_cast<const uint4*>(z + lead) + v0;
+    uint4 v[kU];
+    if (n == 32 * kU) {
+#pragma unroll
+      for (int u = 0; u < kU; ++u) v[u] = load_stream(vp + lane + 32 * u);
+    } else {
+#pragma unroll
+      for (int u = 0; u < kU; ++u) v[u] = load_stream(vp + min(lane + 32 * u, n - 1));
+    }
+    uint32_t packed = packed_max<T>(v[0]);
+#pragma unroll
+    for (int u = 1; u < kU; ++u) packed = packed_max(packed, packed_max<T>(v[u]), T());
+    const float mine = packed_value(packed, T());
+    const float best = warp_max_nan(mine);
+    nan = best != best;
+    unsigned at = 0xffffffffu;  // the lowest index that holds it; with a NaN in the unit none does
+    if (mine == best) {
+      const int first_at = first_holding<T, 0>(v, best);
+      at = lead + (v0 + min(lane + 32 * (first_at / VN), n - 1)) * VN + first_at % VN;
+    }
+    at = __reduce_min_sync(kFull, at);
+    return nan ? 0ull : make_key(best, at);
+  }
+  __device__ __forceinline__ bool has_loose(int V) const {
+    return (first && lead > 0) || (last && lead + nvec * VN < V);
+  }
+  // The loose elements, fewer than VN on either side: one per lane; false in lanes without one.
+  __device__ __forceinline__ bool loose(int V, int lane, float& value, int& at) const {
+    at = lane < VN ? lane : lead + nvec * VN + lane - VN;
+    if (!(lane < VN ? first && at < lead : last && lane < 2 * VN && at < V)) return false;
+    value = Elem<T>::load_cg(z, at);
+    return true;
+  }
+};
+
 // Adds n to its request's counter and runs the selections that this completes
 // (each lane with its own request; lanes with n = 0 add nothing).
 template <typename T, bool kStrict>
@@ -269,9 +244,7 @@ __device__ __noinline__ void count_and_select(const VerifyParams& p, unsigned re
 template <typename T, bool kStrict, bool kSplit, int kU>
 __global__ void __launch_bounds__(kThreads, kSplit ? kStreamMinBlocks : 1)
     verify_stream_kernel(const __grid_constant__ VerifyParams p, const __grid_constant__ StreamPlan q) {
-  constexpr int VN = Elem<T>::kVec;
   const int lane = threadIdx.x & 31;
-  const int V = p.V;
   pdl_signal_dependents();
   if (blockIdx.x < q.draft_ctas) {
     const unsigned row = blockIdx.x * kThreads + threadIdx.x;
@@ -281,8 +254,8 @@ __global__ void __launch_bounds__(kThreads, kSplit ? kStreamMinBlocks : 1)
     bool has_zx = false;
     if (row < q.rows && row - b * (p.K + 1) < static_cast<unsigned>(p.K)) {
       const int x = __ldcg(p.draft + (row - b)) - p.v_offset;  // row = b (K + 1) + j, its draft at b K + j; shard-local
-      has_zx = x >= 0 && x < V;
-      if (has_zx) zx = Elem<T>::load_cg(static_cast<const T*>(p.logits), static_cast<long long>(row) * V + x);
+      has_zx = x >= 0 && x < p.V;
+      if (has_zx) zx = Elem<T>::load_cg(static_cast<const T*>(p.logits), static_cast<long long>(row) * p.V + x);
     }
     pdl_wait_prerequisites();  // resident inputs: before the first touch of the workspace
     if (has_zx) p.draft_logit[row] = zx;
@@ -295,76 +268,38 @@ __global__ void __launch_bounds__(kThreads, kSplit ? kStreamMinBlocks : 1)
   const unsigned unit = (blockIdx.x - q.draft_ctas) * kWarpsPerBlock + warp;
   const unsigned row = q.by_units(unit);
   const int k = static_cast<int>(unit - row * q.units);
-  // The row's elements: loose ones up to the first 16-byte boundary, nvec whole
-  // vectors, loose ones again. Units meet on 128-byte lines, so that a line is
-  // read by one load of one warp.
-  const long long row0 = static_cast<long long>(row) * V;
-  const long long past = row0 - p.head;
-  int lead = static_cast<int>(past <= 0 ? -past : -past & (VN - 1));
-  lead = lead < V ? lead : V;
-  const int nvec = (V - lead) / VN;
-  const int line = static_cast<int>((past + lead) / VN + q.line) & 7;
-  const bool first = k == 0, last = k == q.units - 1;
-  const int v0 = first ? 0 : min(k * q.per - line, nvec);
-  const int v1 = last ? nvec : min((k + 1) * q.per - line, nvec);
-  const T* z = static_cast<const T*>(p.logits) + row0;
+  const Unit<T> mine(p, row, k, q.units, q.per, q.line);
 
   // The logits may be the previous kernel's unless the caller declared them
   // resident; the workspace is touched after the wait below.
   if (!p.resident) pdl_wait_prerequisites();
-  const bool mine_exists = unit < q.total;
-  const int n = v1 - v0;
+  const bool exists = unit < q.total;
   unsigned long long key = 0ull;
-  if (mine_exists && n > 0) {
-    // past its end a unit repeats its last vector, which changes no maximum and no index
-    const uint4* vp = reinterpret_cast<const uint4*>(z + lead) + v0;
-    uint4 v[kU];
-    if (n == 32 * kU) {
-#pragma unroll
-      for (int u = 0; u < kU; ++u) v[u] = load_stream(vp + lane + 32 * u);
-    } else {
-#pragma unroll
-      for (int u = 0; u < kU; ++u) v[u] = load_stream(vp + min(lane + 32 * u, n - 1));
-    }
-    uint32_t packed = packed_max<T>(v[0]);
-#pragma unroll
-    for (int u = 1; u < kU; ++u) packed = packed_max(packed, packed_max<T>(v[u]), T());
-    const float mine = packed_value(packed, T());
-    const float best = warp_max_nan(mine);
-    unsigned at = 0xffffffffu;  // the lowest index that holds it; with a NaN in the unit none does
-    if (mine == best) {
-      const int first_at = first_holding<T, 0>(v, best);
-      at = lead + (v0 + min(lane + 32 * (first_at / VN), n - 1)) * VN + first_at % VN;
-    }
-    at = __reduce_min_sync(kFull, at);
-    if (best == best) {
-      key = make_key(best, at);
-    } else if (lane == 0) {
+  if (exists) {
+    bool nan = false;
+    key = mine.template vectors<kU>(lane, nan);
+    if (nan && lane == 0) {
       pdl_wait_prerequisites();
       atomicOr(&p.flags[q.by_k1(row)], ASD_STATUS_NAN_LOGIT);
     }
-  }
-  if (mine_exists && ((first && lead > 0) || (last && lead + nvec * VN < V))) {
-    // loose elements, fewer than VN on either side: one per lane, each merged by itself
-    pdl_wait_prerequisites();
-    const int e = lane < VN ? lane : lead + nvec * VN + lane - VN;
-    if (lane < VN ? first && e < lead : last && lane < 2 * VN && e < V) {
-      const float loose = Elem<T>::load_cg(z, e);
-      if (loose == loose) {
-        atomicMax(&p.row_key[row], make_key(loose, static_cast<uint32_t>(e)));
-      } else {
-        atomicOr(&p.flags[q.by_k1(row)], ASD_STATUS_NAN_LOGIT);
+    if (mine.has_loose(p.V)) {  // each merged by itself
+      pdl_wait_prerequisites();
+      float value;
+      int at;
+      if (mine.loose(p.V, lane, value, at)) {
+        if (value == value) {
+          atomicMax(&p.row_key[row], make_key(value, static_cast<uint32_t>(at)));
+        } else {
+          atomicOr(&p.flags[q.by_k1(row)], ASD_STATUS_NAN_LOGIT);
+        }
       }
     }
   }
   // one reduction per row and CTA
   if (lane == 0) {
     s_key[warp] = key;
-    s_row[warp] = mine_exists ? row : 0xffffffffu;
-    if (!kSplit) {
-      const int rel0 = first ? 0 : lead + v0 * VN, rel1 = last ? V : lead + v1 * VN;
-      s_count[warp] = mine_exists ? static_cast<unsigned>(rel1 - rel0) : 0u;
-    }
+    s_row[warp] = exists ? row : 0xffffffffu;
+    if (!kSplit) s_count[warp] = exists ? static_cast<unsigned>(mine.elements(p.V)) : 0u;
   }
   if (!kSplit) __threadfence();
   pdl_wait_prerequisites();  // resident inputs: before the first touch of the workspace
@@ -384,86 +319,130 @@ __global__ void __launch_bounds__(kThreads, kSplit ? kStreamMinBlocks : 1)
                                  lane < kWarpsPerBlock ? s_count[lane] : 0u, lane);
 }
 
-// ---------------------------------------------------------------- one CTA per request (small inputs)
+// ---------------------------------------------------------------- one CTA or one cluster per request
 //
-// When a request's K+1 rows are a few KB, what the streaming kernels pay for is
-// their global round trips (row keys, counters, fences), not the bytes. Here a
-// CTA takes one request: its warps split the request's rows flatly (one round
-// of loads, every lane with up to kSmallUnroll vectors in flight), merge the
-// row keys and the draft logits in shared memory, and warp 0 runs Alg. 1 from
-// there. The workspace is not touched.
+// When a request's K+1 rows are few KB, what the streaming kernels pay for is
+// their global round trips (row keys, counters, the hand-off to the selection),
+// not the bytes. Here the CTAs of one cluster take one request: their warps
+// split its rows flatly (one round of loads, every lane with up to kSmallUnroll
+// vectors in flight) and merge the row keys in shared memory, the other CTAs hand
+// theirs to the first one, and its warp 0 runs Alg. 1; lane j of that warp has
+// fetched row j's draft token and its logit meanwhile. The workspace is not touched.
 
 constexpr int kSmallThreads = 512;
 constexpr int kSmallUnroll = 8;
-constexpr long long kSmallMaxRequestBytes = 16LL * kSmallThreads * kSmallUnroll;  // 64 KB: one round of loads
+constexpr long long kSmallCtaBytes = 16LL * kSmallThreads * kSmallUnroll;  // 64 KB: one round of loads
+constexpr int kSmallMaxCluster = 8;                                        // the largest portable cluster
 
-template <typename T, bool kStrict>
-__global__ void __launch_bounds__(kSmallThreads) verify_small_kernel(const __grid_constant__ VerifyParams p) {
+__device__ __forceinline__ uint32_t first_cta_address(const void* smem) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(smem)));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+struct SmallPlan {
+  int units;  // units per row
+  int per;    // vectors per unit, a multiple of 32
+  int line;   // where in its 128-byte line the first vector of the logits lies
+};
+
+template <typename T, bool kStrict, bool kCluster>
+__global__ void __launch_bounds__(kSmallThreads, 1)
+    verify_small_kernel(const __grid_constant__ VerifyParams p, const __grid_constant__ SmallPlan q) {
   __shared__ unsigned long long s_key[32];
-  __shared__ float s_zx[32];
   __shared__ unsigned int s_flags;
-  constexpr int VN = Elem<T>::kVec;
-  constexpr int kWarps = kSmallThreads / 32;
-  const int b = blockIdx.x;
+  __shared__ unsigned long long s_peer_key[kCluster ? kSmallMaxCluster : 1][32];  // first CTA: what the others found
+  __shared__ unsigned int s_peer_flags[kCluster ? kSmallMaxCluster : 1];
+  unsigned rank = 0, ctas = 1;
+  if (kCluster) {
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(ctas));
+  }
+  const int b = blockIdx.x / ctas;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int V = p.V, K = p.K, K1 = p.K + 1;
-  if (threadIdx.x < 32) {
-    s_key[threadIdx.x] = 0ull;
-    s_zx[threadIdx.x] = 0.0f;
-  }
+  const bool selects = rank == 0 && warp == 0;
+  if (threadIdx.x < 32) s_key[threadIdx.x] = 0ull;
   if (threadIdx.x == 0) s_flags = 0u;
+  if (kCluster) cluster_arrive();  // this CTA has started, its shared memory can be written
   // Programmatic dependent launch: the next call's CTAs may start now. With
   // resident inputs this call reads its logits and drafts before the previous
   // kernel on the stream has completed; the ledger and the outputs, which that
   // kernel may use, wait for it in every case.
   pdl_signal_dependents();
   if (!p.resident) pdl_wait_prerequisites();
-  float budget = 0.0f, spent = 0.0f;
-  if (!kStrict && !p.resident && threadIdx.x == 0) {  // in flight while the logits stream
-    budget = p.ledger[b].budget;
-    spent = p.ledger[b].spent;
+  const T* z = static_cast<const T*>(p.logits);
+  float budget = 0.0f, spent = 0.0f, zx = 0.0f;
+  int x = -1;
+  if (selects) {  // in flight while the logits stream
+    if (!kStrict && !p.resident && lane == 0) {
+      budget = __ldcg(&p.ledger[b].budget);
+      spent = __ldcg(&p.ledger[b].spent);
+    }
+    if (lane < K) x = __ldcg(p.draft + static_cast<long long>(b) * K + lane);
   }
   __syncthreads();
 
-  const T* z = static_cast<const T*>(p.logits);
-  const long long n = static_cast<long long>(K1) * V;
-  const long long base = static_cast<long long>(b) * n;
-  long long per = (n + kWarps - 1) / kWarps;
-  per = (per + VN - 1) / VN * VN;
-  const long long lo = base + (warp * per < n ? warp * per : n);
-  const long long hi = base + ((warp + 1) * per < n ? (warp + 1) * per : n);
-  for (long long s0 = lo; s0 < hi;) {
-    const long long row = s0 / V;
-    const long long row0 = row * V;
-    const long long s1 = hi < row0 + V ? hi : row0 + V;
-    const int j = static_cast<int>(row - static_cast<long long>(b) * K1);
-    bool nan = false;
-    const unsigned long long key = segment_key<T, kSmallUnroll>(z, s0, s1, row0, p.head, lane, &nan);
-    if (lane == 0) {
-      atomicMax(&s_key[j], key);
-      if (nan) atomicOr(&s_flags, ASD_STATUS_NAN_LOGIT);
-      if (j < K) {
-        const int x = __ldg(p.draft + static_cast<long long>(b) * K + j);
-        if (x >= 0 && x < V && row0 + x >= s0 && row0 + x < s1) s_zx[j] = Elem<T>::load(z, row0 + x);
-      }
-    }
-    s0 = s1;
+  // Warp 0 of the first CTA fetches the drafts' logits, the others share the
+  // request's units.
+  bool nan = false;
+  if (selects) {
+    if (x >= 0 && x < V) zx = Elem<T>::load_cg(z, (static_cast<long long>(b) * K1 + lane) * V + x);
   }
+  const int warps = (kSmallThreads / 32) * static_cast<int>(ctas) - 1;
+  for (int u = static_cast<int>(rank) * (kSmallThreads / 32) + warp - 1; !selects && u < K1 * q.units; u += warps) {
+    const int j = u / q.units;
+    const Unit<T> unit(p, static_cast<long long>(b) * K1 + j, u - j * q.units, q.units, q.per, q.line);
+    bool unit_nan = false;
+    const unsigned long long key = unit.template vectors<kSmallUnroll>(lane, unit_nan);
+    nan |= unit_nan;
+    if (lane == 0 && key) atomicMax(&s_key[j], key);
+    if (unit.has_loose(V)) {
+      float value;
+      int at;
+      const bool has = unit.loose(V, lane, value, at);
+      if (has && value == value) atomicMax(&s_key[j], make_key(value, static_cast<uint32_t>(at)));
+      nan |= __any_sync(kFull, has && value != value);
+    }
+  }
+  if (nan && lane == 0) atomicOr(&s_flags, ASD_STATUS_NAN_LOGIT);
   __syncthreads();
-  if (warp != 0) return;
+  if (kCluster) {
+    cluster_wait();  // the first CTA has started
+    if (rank != 0 && warp == 0) {
+      if (lane < K1)
+        asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(first_cta_address(&s_peer_key[rank][lane])), "l"(s_key[lane])
+                     : "memory");
+      if (lane == 0)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(first_cta_address(&s_peer_flags[rank])), "r"(s_flags) : "memory");
+      __syncwarp();
+    }
+    cluster_arrive();
+    cluster_wait();
+  }
+  if (!selects) return;
   if (p.resident) {
     pdl_wait_prerequisites();
     if (!kStrict && lane == 0) {
-      budget = p.ledger[b].budget;
-      spent = p.ledger[b].spent;
+      budget = __ldcg(&p.ledger[b].budget);
+      spent = __ldcg(&p.ledger[b].spent);
     }
   }
 
   BlockInputs in;
   in.key = lane < K1 ? s_key[lane] : 0ull;
-  in.x = lane < K ? __ldg(p.draft + static_cast<long long>(b) * K + lane) : -1;
-  in.zx = lane < K ? s_zx[lane] : 0.0f;
+  in.x = x;
+  in.zx = zx;
   in.flags = s_flags | workspace_failed(p, lane);
+  if (kCluster) {
+    for (unsigned i = 1; i < ctas; ++i) {
+      const unsigned long long o = lane < K1 ? s_peer_key[i][lane] : 0ull;
+      in.key = o > in.key ? o : in.key;
+      in.flags |= s_peer_flags[i];
+    }
+  }
   in.top = ordered_value(static_cast<uint32_t>(in.key >> 32));
   in.top_exact = false;
   budget = __shfl_sync(kFull, budget, 0);
@@ -1062,33 +1041,61 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
 //            A slice pays for every row it enters: at 200 MB the two meet
 //            between 100 KB rows (35.6 against 31.7 us) and 128 KB rows (30.0
 //            against 31.1 us).
-//   kSmall   one CTA per request, below kTmaMinBytes, when a request fits one
-//            round of loads of a CTA (single blocks, no vocabulary shard).
+//   kSmall   a request fits one round of loads of a cluster (508 KB; 60 KB for
+//            one CTA) and there are few enough: no hand-off to a selection, one
+//            launch. With one CTA each 2.4 against 3.0 us (8 requests of 18 KB),
+//            3.0 against 5.1 (152 of 18 KB), 4.8 against 6.0 us (128 of 54 KB).
+//            With a cluster 3.5 against 4.2 us (16 of 144 KB), no gain for one
+//            call alone that waits (3.25 us both, 2 of 320 KB) but half the
+//            launches, and 1.5 against 2.5 us with resident inputs. A GPU full of
+//            clusters of four or eight is slower: 7.2 against 5.7 us (19 of 504
+//            KB), 6.9 against 5.0 us (38 of 216 KB).
 //   kStream  everything else. A call that waits for the kernel ahead of it has
 //            nothing to overlap and takes 15.5 us for 87.5 MB where the TMA
 //            pipeline took 20.5 us, 93 against 100 us for 662 MB, 4.0 against
-//            8.2 us for 2.7 MB, 7.4 against 26 us for 16 MB in 2 KB rows.
+//            8.2 us for 2.7 MB, 7.0 against 26 us for 16 MB in 2 KB rows.
 // The launch options can force a kernel (the tests use that to cover every
 // kernel); a forced `small` falls back to the default when the shape does not
 // qualify.
 constexpr long long kTmaMinBytes = 1LL << 20;
 constexpr long long kTmaMinRowBytes = 112LL << 10;
+constexpr long long kSmallMaxBytes = 1LL << 20;         // below this any number of one-CTA requests
+constexpr int kSmallMaxCtas = 304;                      // two a SM
+constexpr int kSmallMaxClusterCtas = 152;
+constexpr long long kSmallMaxClusterBytes = 5LL << 20;  // of clusters larger than two
 
 enum class Path { kSmall, kStream, kTma };
 
-Path choose_path(int forced, long long bytes, long long request_bytes, int K, bool single_block, bool resident) {
-  const bool small_ok = single_block && K + 1 <= 32 && request_bytes <= kSmallMaxRequestBytes;
+// CTAs that take one request together: every lane's share in one round of loads
+// (0: too large).
+int small_cluster(long long request_bytes) {
+  for (int ctas = 1; ctas <= kSmallMaxCluster; ctas *= 2)
+    if (request_bytes <= ctas * kSmallCtaBytes - kSmallCtaBytes / (kSmallThreads / 32)) return ctas;
+  return 0;
+}
+
+Path choose_path(int forced, long long bytes, long long request_bytes, int B, int K, bool single_block, bool resident) {
+  const int ctas = single_block ? small_cluster(request_bytes) : 0;
   if (forced == ASD_PATH_TMA) return Path::kTma;
   if (forced == ASD_PATH_STREAM) return Path::kStream;
-  if (forced == ASD_PATH_SMALL && small_ok) return Path::kSmall;
-  if (bytes < kTmaMinBytes) return small_ok ? Path::kSmall : Path::kStream;
-  return resident && request_bytes / (K + 1) >= kTmaMinRowBytes ? Path::kTma : Path::kStream;
+  if (forced == ASD_PATH_SMALL && ctas > 0) return Path::kSmall;
+  if (ctas == 1 && (bytes < kSmallMaxBytes || B <= kSmallMaxCtas)) return Path::kSmall;
+  if (ctas > 1 && static_cast<long long>(B) * ctas <= kSmallMaxClusterCtas &&
+      (ctas == 2 || bytes <= kSmallMaxClusterBytes))
+    return Path::kSmall;
+  return resident && bytes >= kTmaMinBytes && request_bytes / (K + 1) >= kTmaMinRowBytes ? Path::kTma : Path::kStream;
 }
 
 // The cut of a row into units: as large as a warp's loads in flight allow, but
 // no larger than spreads a small input over kStreamWarpsPerSm warps on every SM.
 constexpr int kStreamWarpsPerSm = 16;
 constexpr long long kStreamMaxUnits = 1LL << 31;  // unit numbers are 32-bit
+
+// Where in its 128-byte line the logits' first whole vector lies.
+template <typename T>
+int first_line(const VerifyParams& p) {
+  return static_cast<int>((reinterpret_cast<uintptr_t>(p.logits) + static_cast<size_t>(p.head) * sizeof(T)) / 16 % 8);
+}
 
 template <typename T>
 StreamPlan stream_plan(const VerifyParams& p, long long rows, int sms) {
@@ -1099,7 +1106,7 @@ StreamPlan stream_plan(const VerifyParams& p, long long rows, int sms) {
   per = per < 32 ? 32 : per > 32 * kStreamUnroll ? 32 * kStreamUnroll : per;
   q.per = static_cast<int>(per);
   q.units = nvec <= per ? 1 : static_cast<int>((nvec + 7 + per - 1) / per);  // + 7: the first unit may begin inside a line
-  q.line = static_cast<int>((reinterpret_cast<uintptr_t>(p.logits) + static_cast<size_t>(p.head) * sizeof(T)) / 16 % 8);
+  q.line = first_line<T>(p);
   q.rows = static_cast<unsigned>(rows);
   q.by_units.set(static_cast<unsigned>(q.units));
   q.by_k1.set(static_cast<unsigned>(p.K + 1));
@@ -1136,10 +1143,41 @@ int launch_stream(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream
 }
 
 template <typename T, bool kStrict>
+int launch_small(const VerifyParams& p, int ctas, const LaunchOptions& opt, cudaStream_t stream) {
+  SmallPlan q;
+  const int nvec = p.V / Elem<T>::kVec;                                // whole vectors of a row, at most
+  const int warps = ctas * (kSmallThreads / 32) - 1;                   // one fetches the drafts' logits
+  const int share = warps / (p.K + 1) > 0 ? warps / (p.K + 1) : 1;     // units per row that start at once
+  q.per = ((nvec + 7 + share - 1) / share + 31) / 32 * 32;
+  if (q.per > 32 * kSmallUnroll) q.per = 32 * kSmallUnroll;
+  q.units = nvec <= q.per ? 1 : (nvec + 7 + q.per - 1) / q.per;  // + 7: the first unit may begin inside a line
+  q.line = first_line<T>(p);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(p.B) * static_cast<unsigned>(ctas));
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  if (opt.pdl) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (ctas > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = static_cast<unsigned>(ctas);
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  auto kernel = ctas > 1 ? verify_small_kernel<T, kStrict, true> : verify_small_kernel<T, kStrict, false>;
+  if (cudaLaunchKernelEx(&cfg, kernel, p, q) != cudaSuccess) return ASD_ERR_CUDA;
+  return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+}
+
+template <typename T, bool kStrict>
 int launch(VerifyParams& p, cudaStream_t stream) {
   const long long request_bytes = static_cast<long long>(p.K + 1) * p.V * static_cast<long long>(sizeof(T));
   const LaunchOptions opt = launch_options();
-  const Path path = choose_path(opt.path, p.total * static_cast<long long>(sizeof(T)), request_bytes, p.K,
+  const Path path = choose_path(opt.path, p.total * static_cast<long long>(sizeof(T)), request_bytes, p.B, p.K,
                                 p.nblk == 1 && !p.partials, p.resident != 0);
   if (path == Path::kTma) return launch_tma<T, kStrict>(p, opt, stream);
   const uintptr_t addr = reinterpret_cast<uintptr_t>(p.logits);
@@ -1148,19 +1186,7 @@ int launch(VerifyParams& p, cudaStream_t stream) {
   if (head > p.total) head = p.total;
   if (path == Path::kSmall) {
     p.head = head;
-      cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(p.B));
-    cfg.blockDim = dim3(kSmallThreads);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    if (opt.pdl) {
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-    }
-    if (cudaLaunchKernelEx(&cfg, verify_small_kernel<T, kStrict>, p) != cudaSuccess) return ASD_ERR_CUDA;
-    return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+    return launch_small<T, kStrict>(p, small_cluster(request_bytes), opt, stream);
   }
   p.head = head;
   return opt.split ? launch_stream<T, kStrict, true>(p, opt, stream) : launch_stream<T, kStrict, false>(p, opt, stream);
@@ -1289,7 +1315,7 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches) {
   if (rc != ASD_OK) return rc;
   const long long request_bytes = static_cast<long long>(K + 1) * V * (dtype_code(dtype) == ASD_BF16 ? 2 : 4);
   const LaunchOptions opt = launch_options();
-  const Path path = choose_path(opt.path, request_bytes * B, request_bytes, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0);
+  const Path path = choose_path(opt.path, request_bytes * B, request_bytes, B, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0);
   *launches = B == 0 ? 0 : (path != Path::kSmall && opt.split ? 2 : 1);
   return ASD_OK;
 }

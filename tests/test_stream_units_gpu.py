@@ -1,7 +1,7 @@
-"""The register-streaming row stage at the sizes where its cut of a row into units can go wrong: one vector
+"""The row stages that cut rows into units, at the sizes where its cut of a row into units can go wrong: one vector
 either side of a unit, a unit of one, four and eight loads per lane, rows shorter than a vector, starts off the
 16-byte and the 128-byte grid, rows whose maximum sits at a unit's edge or is tied across units, rows of -inf,
-infinities and the lowest finite value. Every output bit for bit the oracle's (comparisons and one fp32
+infinities and the lowest finite value; requests on both sides of each cluster size. Every output bit for bit the oracle's (comparisons and one fp32
 subtraction decide all of them)."""
 import math
 
@@ -76,3 +76,41 @@ def test_both_sides_of_the_dispatch(asd, row_bytes, resident):
         torch.cuda.synchronize()
         want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), math.inf, 2)
         _equal(out, want, f"V={V} B={B}")
+
+
+@pytest.mark.parametrize("resident", [False, True])
+@pytest.mark.parametrize("K", [0, 8, 31])
+@pytest.mark.parametrize("ctas", [1, 2, 4, 8])
+def test_request_clusters(asd, ctas, K, resident):
+    """Requests that just fill, and just do not fill, one round of loads of a cluster of each size; a NaN in
+    one request flags that request only, whichever CTA of its cluster meets it."""
+    limit = ctas * 65536 - 4096
+    for dtype, size in ((torch.bfloat16, 2), (torch.float32, 4)):
+        for V in (limit // size // (K + 1), limit // size // (K + 1) + 1):
+            B = 5
+            off = (V + K) % 8
+            flat = torch.randn(off + B * (K + 1) * V, device="cuda").mul_(3.0).to(dtype)
+            z = flat[off:].view(B, K + 1, V)
+            for j in range(K + 1):
+                z[0, j, (j * V) // (K + 1)] = 40.0
+                z[1, j, V - 1 - j] = 40.0
+            z[2, K, V - 1] = math.nan
+            z[3, 0, 0] = math.nan
+            draft = torch.randint(0, V, (B, K), dtype=torch.int32, device="cuda")
+            if K:
+                draft[:2] = z[:2, :K].float().argmax(2).to(torch.int32)
+            ledger = asd.make_ledger(B, 8.0)
+            torch.cuda.synchronize()
+            try:
+                asd.set_launch_options(path="small")
+                out = asd.verify(z, draft, ledger, 1.0, 2, resident=resident)
+                torch.cuda.synchronize()
+            finally:
+                asd.reset_launch_options()
+            want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), 1.0, 2)
+            assert np.array_equal(out["status"].cpu().numpy(), want["status"])
+            clean = want["status"] == 0
+            assert clean.tolist() == [True, True, False, False, True]
+            got = {k: v[torch.from_numpy(clean).cuda()] for k, v in out.items()}
+            _equal(got, {k: v[clean] for k, v in want.items() if k != "ledger"}, f"V={V} off={off} {dtype}")
+            assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
