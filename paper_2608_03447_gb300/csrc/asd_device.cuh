@@ -135,21 +135,22 @@ __device__ __forceinline__ BlockInputs load_block(const VerifyParams& p, long lo
   in.x = -1;
   in.zx = 0.0f;
   in.flags = 0;
-  if (lane < K1) {
-    in.key = __ldcg(&p.row_key[row]);
-    p.row_key[row] = 0ull;  // the whole workspace is zero again after every call
-  }
+  if (lane < K1) in.key = __ldcg(&p.row_key[row]);
   if (lane < K) {
     in.x = __ldcg(p.draft + vb * K + lane);
     in.zx = __ldcg(&p.draft_logit[row]);
-    p.draft_logit[row] = 0.0f;
   }
   if (lane == 0) {
     const unsigned f = __ldcg(&p.flags[vb]);
     const unsigned e = (kWithError && p.error) ? __ldcg(p.error) : 0u;
-    p.flags[vb] = 0u;
     in.flags = f | (e ? ASD_STATUS_INCOMPLETE : 0u);
   }
+  // the whole workspace is zero again after every call; the compiler must not
+  // move these stores ahead of the loads, which it does not know to be loads
+  asm volatile("" ::: "memory");
+  if (lane < K1) p.row_key[row] = 0ull;
+  if (lane < K) p.draft_logit[row] = 0.0f;
+  if (lane == 0) p.flags[vb] = 0u;
   in.flags = __shfl_sync(kFull, in.flags, 0);
   in.top = ordered_value(static_cast<uint32_t>(in.key >> 32));
   in.top_exact = false;
@@ -180,7 +181,8 @@ __device__ __forceinline__ void select_block(const VerifyParams& p, long long vb
   if (lane < K) {
     if (valid_x) {
       float t = top;
-      if (t == 0.0f && !in.top_exact && z) t = Elem<T>::load(z, row * p.V + y);
+      if (t == 0.0f && !in.top_exact && z && static_cast<unsigned>(y) < static_cast<unsigned>(p.V))
+        t = Elem<T>::load(z, row * p.V + y);
       r = __fsub_rn(t, in.zx);
     } else {
       r = __int_as_float(0x7fc00000);
@@ -259,7 +261,7 @@ __device__ void emit_partials(const VerifyParams& p, int b, int lane) {
     const long long row = static_cast<long long>(b) * K1 + lane;
     const uint32_t local = 0xffffffffu - static_cast<uint32_t>(in.key);
     float top = in.top;
-    if (top == 0.0f && in.key && z) top = Elem<T>::load(z, row * p.V + local);  // keep the sign of a zero
+    if (top == 0.0f && local < static_cast<uint32_t>(p.V) && z) top = Elem<T>::load(z, row * p.V + local);  // keep the sign of a zero
     const int xl = lane < K ? in.x - p.v_offset : -1;
     asd_partial out;
     out.key = in.key ? ((in.key & 0xffffffff00000000ull) |

@@ -138,12 +138,6 @@ __device__ __forceinline__ uint32_t packed_max(const uint4& v) {
   return packed_max(packed_max(v.x, v.y, T()), packed_max(v.z, v.w, T()), T());
 }
 
-__device__ __forceinline__ float warp_max_nan(float v) {
-  float m;
-  asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
-  return m;
-}
-
 // VN u + t: element t of v[u] is the first that equals best, one of them does.
 template <typename T, int u, int kU>
 __device__ __forceinline__ int first_holding(const uint4 (&v)[kU], float best) {
@@ -202,15 +196,16 @@ struct Unit {
 #pragma unroll
     for (int u = 1; u < kU; ++u) packed = packed_max(packed, packed_max<T>(v[u]), T());
     const float mine = packed_value(packed, T());
-    const float best = warp_max_nan(mine);
-    nan = best != best;
-    unsigned at = 0xffffffffu;  // the lowest index that holds it; with a NaN in the unit none does
-    if (mine == best) {
-      const int first_at = first_holding<T, 0>(v, best);
+    nan = __any_sync(kFull, mine != mine);
+    const uint32_t order = ordered_bits(mine);
+    const uint32_t best = __reduce_max_sync(kFull, order);
+    unsigned at = 0xffffffffu;  // the lowest index that holds it
+    if (order == best) {
+      const int first_at = first_holding<T, 0>(v, mine);
       at = lead + (v0 + min(lane + 32 * (first_at / VN), n - 1)) * VN + first_at % VN;
     }
     at = __reduce_min_sync(kFull, at);
-    return nan ? 0ull : make_key(best, at);
+    return nan ? 0ull : (static_cast<unsigned long long>(best) << 32) | (0xffffffffu - at);
   }
   __device__ __forceinline__ bool has_loose(int V) const {
     return (first && lead > 0) || (last && lead + nvec * VN < V);

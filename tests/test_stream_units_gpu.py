@@ -34,7 +34,7 @@ def test_unit_edges(asd, dtype, vectors, fused):
         if V < 1:
             continue
         K = 3
-        B = max(2, (rows_mb << 20) // ((K + 1) * V * (16 // vn)))
+        B = max(3, (rows_mb << 20) // ((K + 1) * V * (16 // vn)))
         if B * (K + 1) > 6000:
             continue  # the longer rows cover this
         off = int(rng.integers(0, 64))
@@ -47,6 +47,9 @@ def test_unit_edges(asd, dtype, vectors, fused):
         z[1, 1, [V - 1, V // 2]] = 50.0                      # a tie: the lower index
         z[1, 2, V // 3] = math.inf
         z[1, 3] = torch.finfo(dtype).min
+        z[2, 0] = -1.0
+        z[2, 0, V // 2] = 1e-39                              # subnormal maxima
+        z[2, 1] = -1e-39
         draft = torch.randint(0, V, (B, K), dtype=torch.int32, device="cuda")
         draft[:, 0] = z[:, 0].argmax(1)                      # the tops among the drafts, so longer prefixes occur
         ledger = asd.make_ledger(B, 8.0)
