@@ -117,3 +117,30 @@ def test_request_clusters(asd, ctas, K, resident):
             got = {k: v[torch.from_numpy(clean).cuda()] for k, v in out.items()}
             _equal(got, {k: v[clean] for k, v in want.items() if k != "ledger"}, f"V={V} off={off} {dtype}")
             assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
+
+
+@pytest.mark.parametrize("nblk", [2, 7, 8, 9, 17])
+def test_blocks_around_the_warps_of_a_selection(asd, nblk):
+    """The ledger goes through fewer, as many and more blocks than the selection's CTA has warps; one block in
+    the middle of a request has a NaN, an out-of-range draft sits in the last."""
+    B, K, V = 5, 6, 4001
+    z = torch.randn(nblk, B, K + 1, V, device="cuda").mul_(3.0).to(torch.bfloat16)
+    draft = z[:, :, :K].float().argmax(3).to(torch.int32)
+    near = torch.rand(nblk, B, K, device="cuda") < 0.4
+    second = z[:, :, :K].float().topk(2, dim=3).indices[..., 1].to(torch.int32)
+    draft = torch.where(near, second, draft).contiguous()
+    z[nblk // 2, 1, 0, 7] = math.nan
+    draft[nblk - 1, 2, 0] = V
+    ledger = asd.make_ledger(B, 6.0)
+    torch.cuda.synchronize()
+    out = asd.verify_blocks(z, draft, ledger, 1.0, 3)
+    torch.cuda.synchronize()
+    want_ledger = np.array([[6.0, 0.0]] * B, np.float32)
+    for i in range(nblk):
+        want = oracle.verify(z[i].cpu(), draft[i].cpu().numpy(), want_ledger, 1.0, 3)
+        want_ledger = want["ledger"]
+        assert np.array_equal(out["status"][i].cpu().numpy(), want["status"])
+        ok = torch.from_numpy((want["status"] & oracle.STATUS_NAN_LOGIT) == 0)
+        _equal({k: v[i][ok.cuda()] for k, v in out.items()},
+               {k: v[ok.numpy()] for k, v in want.items() if k != "ledger"}, f"block {i}")
+    assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want_ledger.view(np.uint32))
