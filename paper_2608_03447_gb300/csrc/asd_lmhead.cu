@@ -21,7 +21,7 @@
 // Per CTA: warp 0 issues TMA loads (128B-swizzled 64-wide K slabs) into a ring
 // of as many stages as fit, whose completion is counted on the first CTA's
 // barrier; warp 1 allocates tensor memory, and in the first CTA one of its
-// threads issues the MMAs; warps 2-9 reduce the accumulators. Accumulators are
+// threads issues the MMAs; the other warps reduce the accumulators. Accumulators are
 // slots in a ring of two to four (512 columns / token tile width), each handed
 // over by barriers of its own, so that the MMAs of the next item begin when one
 // tile has been read and run ahead in it while the other is being read.
@@ -57,8 +57,16 @@ constexpr int kMaxStages = 6;
 constexpr int kSlabA = kHalfM * kBK * 2;  // 16 KB of vocabulary rows per tile
 constexpr int kStageA = kW * kSlabA;
 constexpr int kMaxSlots = 4;              // accumulators in tensor memory
-constexpr int kEpiWarps = 8;              // two per TMEM lane quarter, 32-column blocks alternating
-constexpr int kLmThreads = (2 + kEpiWarps) * 32;  // producer, MMA, epilogue warps
+// Epilogue warps: a tile's 32-column blocks go in turn to the warps of each TMEM
+// lane quarter. A reduction that still has to look for its maxima (a pair's first
+// item) takes 1.2 us a block, and nothing hides it behind a pair's last item. With
+// one token tile, where that is what a call adds to streaming the weight, there are
+// sixteen warps instead of eight: 256 tokens on a 38912-row shard 73.5 us instead of
+// 77.2, 160 tokens 68.5 instead of 70.8, 18 tokens 65.3 instead of 65.7. With more
+// tiles (or logits to write) the tensor cores set the pace, and sixteen gain nothing.
+constexpr int kEpiWarpsOneTile = 16;
+constexpr int kEpiWarps = 8;
+constexpr int lm_threads(int epi_warps) { return (2 + epi_warps) * 32; }  // producer, MMA, epilogue warps
 constexpr int kTmemCols = 512;
 static_assert(kEpiWarps * 32 >= kMaxTN, "one epilogue thread per token column");
 
@@ -284,9 +292,10 @@ __device__ __forceinline__ void abort_pair(LmShared& sh, uint32_t peer) {
 // whatever its sign bit, so a NaN anywhere in a row reaches the row's key.
 __device__ __forceinline__ uint32_t max_bits(float v) { return v != v ? 0xffc00000u : ordered_bits(v); }
 
-// Meets the kThreads threads of the epilogue warps.
+// Meets the threads of the epilogue warps.
+template <int kEpi>
 __device__ __forceinline__ void epilogue_sync() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+  asm volatile("bar.sync 1, %0;" ::"n"(kEpi * 32) : "memory");
 }
 
 // Argmax of one warp's 32 x 32 block of logits: vocabulary rows v_warp on (TMEM
@@ -421,8 +430,8 @@ __device__ __forceinline__ LmItem lm_item(const LmParams& q, int entry) {
 }
 
 // One CTA pair (cluster of 2) works through entries pair, pair + pairs, ...
-template <bool kWriteLogits>
-__global__ void __launch_bounds__(kLmThreads, 1)
+template <bool kWriteLogits, int kEpi>
+__global__ void __launch_bounds__(lm_threads(kEpi), 1)
     lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w,
                          const __grid_constant__ VerifyParams p, const __grid_constant__ LmParams q) {
   extern __shared__ __align__(1024) unsigned char lm_smem_raw[];
@@ -451,7 +460,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
     }
     for (int s = 0; s < kMaxSlots; ++s) {
       mbar_init(&sh.acc_full[s], 1);
-      mbar_init(&sh.acc_empty[s], 2 * kEpiWarps);  // the epilogue warps of both CTAs
+      mbar_init(&sh.acc_empty[s], 2 * kEpi);  // the epilogue warps of both CTAs
     }
     mbar_init(&sh.drain, 1);
     sh.abort = 0;
@@ -608,10 +617,13 @@ __global__ void __launch_bounds__(kLmThreads, 1)
       __syncwarp();
     }
   } else {
-    // ---------------- epilogue: warps 2-9, one TMEM lane quarter each; the two warps of a quarter take
-    // alternate 32-column blocks of every accumulator
-    const int quarter = warp & 3;                     // TMEM lanes this warp may read
-    const int c_first = ((warp - 2) >> 2) * 32;
+    // ---------------- epilogue: warps 2 on, each on one TMEM lane quarter. The warps of a quarter deal its
+    // 32-column blocks in turn; with four, the second tile's on from the first's, so that tiles of few blocks are
+    // read by different warps.
+    constexpr int kTurns = kEpi / 4;
+    const int quarter = warp & 3;  // TMEM lanes this warp may read
+    const int turn = (warp - 2) >> 2;
+    const int blocks = q.tn / 32;
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const uint32_t acc_empty0 = map_rank(smem_u32(&sh.acc_empty[0]), 0);
     const int et = static_cast<int>(threadIdx.x) - 64;  // this thread among the epilogue's: its token column
@@ -639,7 +651,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
           sh.best[et] = known;
           sh.thr[et] = !has_token ? INFINITY : known ? ordered_value(static_cast<uint32_t>(known >> 32)) : -INFINITY;
         }
-        epilogue_sync();
+        epilogue_sync<kEpi>();
       }
       for (int t = 0; t < it.kw; ++t) {
         // after a wait that gave up the warp goes on without reducing: the other warps meet it at the barriers
@@ -655,7 +667,8 @@ __global__ void __launch_bounds__(kLmThreads, 1)
           const uint32_t acc = tmem + lane_base + static_cast<uint32_t>(slot * q.tn);
           const int v_warp = it.row0 + t * kPairM + static_cast<int>(rank) * kHalfM + quarter * 32;
           if (v_warp < q.V) {  // rows past the vocabulary: nothing to reduce
-            for (int c = c_first; c < q.tn; c += 64) {
+            const int c_first = (kTurns == 4 ? (turn + t * (kTurns - blocks % kTurns)) % kTurns : turn) * 32;
+            for (int c = c_first; c < q.tn; c += kTurns * 32) {
               if (kWriteLogits) {
                 const int v = v_warp + lane;  // this thread's vocabulary row
                 uint32_t r[32];
@@ -682,7 +695,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
         }
       }
       if (!kWriteLogits) {
-        epilogue_sync();  // every warp's maxima are in sh.best
+        epilogue_sync<kEpi>();  // every warp's maxima are in sh.best
         if (has_token) {
           const unsigned long long key = sh.best[et];
           if (key != known) {
@@ -755,7 +768,7 @@ struct LmDevice {
   int major = 0, minor = 0;
   // CTA pairs resident at once, per kernel instance (0: not set up yet); the
   // set-up is idempotent, so two threads racing to do it store the same value
-  std::atomic<int> pairs[2] = {};
+  std::atomic<int> pairs[3] = {};
 };
 
 int lm_device(LmDevice** out) {
@@ -776,11 +789,11 @@ int lm_device(LmDevice** out) {
   return ASD_OK;
 }
 
-cudaLaunchConfig_t pair_config(unsigned grid, size_t smem, cudaStream_t stream, cudaLaunchAttribute (&attr)[2],
-                               bool pdl) {
+cudaLaunchConfig_t pair_config(unsigned grid, int threads, size_t smem, cudaStream_t stream,
+                               cudaLaunchAttribute (&attr)[2], bool pdl) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(kLmThreads, 1, 1);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -822,15 +835,15 @@ void lm_plan(int T, int V, int H, int pairs, LmParams* q) {
   q->entries = items + halved;
 }
 
-template <bool kWriteLogits>
-int launch_lmhead(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
-                  cudaStream_t stream) {
+template <bool kWriteLogits, int kEpi>
+int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
+                         cudaStream_t stream) {
   LmDevice* dev = nullptr;
   int rc = lm_device(&dev);
   if (rc != ASD_OK) return rc;
   if (dev->major != 10) return ASD_ERR_DEVICE;  // tcgen05 needs a Blackwell (sm_10x) device
-  auto kernel = lmhead_verify_kernel<kWriteLogits>;
-  std::atomic<int>& resident = dev->pairs[kWriteLogits ? 1 : 0];
+  auto kernel = lmhead_verify_kernel<kWriteLogits, kEpi>;
+  std::atomic<int>& resident = dev->pairs[kWriteLogits ? 1 : kEpi == kEpiWarps ? 0 : 2];
   cudaLaunchAttribute attr[2];
   int pairs = resident.load(std::memory_order_acquire);
   if (pairs == 0) {
@@ -838,7 +851,8 @@ int launch_lmhead(const void* hidden, const void* weight, int H, int T, VerifyPa
         cudaSuccess)
       return ASD_ERR_CUDA;
     // every token tile width leaves room for one CTA per SM
-    cudaLaunchConfig_t probe = pair_config(static_cast<unsigned>(dev->sms & ~1), kLmSmemMax, stream, attr, false);
+    cudaLaunchConfig_t probe =
+        pair_config(static_cast<unsigned>(dev->sms & ~1), lm_threads(kEpi), kLmSmemMax, stream, attr, false);
     if (cudaOccupancyMaxActiveClusters(&pairs, kernel, &probe) != cudaSuccess || pairs < 1) return ASD_ERR_CUDA;
     resident.store(pairs, std::memory_order_release);
   }
@@ -848,10 +862,18 @@ int launch_lmhead(const void* hidden, const void* weight, int H, int T, VerifyPa
   CUtensorMap map_h, map_w;
   if (!make_map(&map_h, hidden, T, H, q.tn / 2) || !make_map(&map_w, weight, p.V, H, kHalfM)) return ASD_ERR_CUDA;
   const unsigned grid = 2u * static_cast<unsigned>(q.entries < pairs ? q.entries : pairs);
-  cudaLaunchConfig_t cfg = pair_config(grid, lm_smem_bytes(q.tn), stream, attr, true);
+  cudaLaunchConfig_t cfg = pair_config(grid, lm_threads(kEpi), lm_smem_bytes(q.tn), stream, attr, true);
   if (cudaLaunchKernelEx(&cfg, kernel, map_h, map_w, p, q) != cudaSuccess) return ASD_ERR_CUDA;
   if (kWriteLogits) return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
   return launch_select<float, false>(p, true, stream);
+}
+
+template <bool kWriteLogits>
+int launch_lmhead(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
+                  cudaStream_t stream) {
+  if (!kWriteLogits && T <= kMaxTN)
+    return launch_lmhead_kernel<kWriteLogits, kEpiWarpsOneTile>(hidden, weight, H, T, p, logits_out, stream);
+  return launch_lmhead_kernel<kWriteLogits, kEpiWarps>(hidden, weight, H, T, p, logits_out, stream);
 }
 
 int check_lm_inputs(const void* hidden, const void* weight, int H) {
