@@ -282,16 +282,17 @@ __device__ void select_request(const VerifyParams& p, int b, int lane) {
     emit_partials<T>(p, b, lane);
     return;
   }
+  // the ledger, the error word and the first block in one round trip
   float budget = 0.0f, spent = 0.0f;
   if (!kStrict && lane == 0) {
     budget = __ldcg(&p.ledger[b].budget);
     spent = __ldcg(&p.ledger[b].spent);
   }
+  bool wrote = false;
+  BlockInputs cur = load_block<true>(p, b, lane);
+  const unsigned incomplete = cur.flags & ASD_STATUS_INCOMPLETE;
   budget = __shfl_sync(kFull, budget, 0);
   spent = __shfl_sync(kFull, spent, 0);
-  const unsigned incomplete = workspace_failed(p, lane);
-  bool wrote = false;
-  BlockInputs cur = load_block(p, b, lane);
   for (int i = 0; i < p.nblk; ++i) {
     const long long vb = static_cast<long long>(i) * p.B + b;
     BlockInputs next = cur;
