@@ -31,8 +31,8 @@ static __global__ void __launch_bounds__(kSelectThreads) select_kernel(const __g
 // many blocks at once; only the walk over a block's mismatches, which needs the
 // ledger as the block before left it, goes from warp to warp. One warp for all of
 // a request's blocks took 0.85 us per block, most of it waiting for its loads:
-// captured, 3 blocks of 23 requests 18.4 -> 16.1 us (15.3 for 69 requests in one
-// block), 23 of 3 35 -> 26 us, 8 of 8 27 -> 23 us.
+// captured, 3 blocks of 23 requests 18.4 -> 16.1 us, 23 of 3 35 -> 26 us, 8 of 8 27
+// -> 23 us (and 15.8, 24.5 and 22.2 us since the walk visits mismatches only).
 constexpr int kSelectBlocksThreads = 256;
 
 template <typename T>

@@ -81,12 +81,12 @@ __device__ __forceinline__ float vec_max(const uint4& v, __nv_bfloat16) {
 // logits instead, a row per thread.
 //
 // Bound by memory: a kernel that only loads the same bytes this way takes 13.3 us
-// for 87.5 MB and 88.5 us for 662 MB where a call, selection included, takes 15.5
-// and 93 us (the TMA pipeline: 20.5 and 100). What else was measured: 2 KB units
-// with twice the warps 16.0 / 93.2 us; every warp reducing to the row's slot by
-// itself 16.3 / 95.6 us (and 18.4 / 108 us with 2 KB units: the slots of
-// neighbouring rows share a line of L2, which takes them one by one); units that
-// do not end on 128-byte lines, 17.2 / 95.5 us.
+// for 87.5 MB and 88.5 us for 662 MB where a call, selection included, takes 14.8
+// to 15.1 and 91.7 us (the TMA pipeline: 20.5 and 100). What else was measured, when
+// this stood at 15.5 / 92.8 us: 2 KB units with twice the warps 16.0 / 93.2 us; every
+// warp reducing to the row's slot by itself 16.3 / 95.6 us (and 18.4 / 108 us with 2
+// KB units: the slots of neighbouring rows share a line of L2, which takes them one
+// by one); units that do not end on 128-byte lines, 17.2 / 95.5 us.
 struct StreamPlan {
   unsigned draft_ctas;  // CTAs that fetch draft logits
   unsigned rows;
@@ -228,7 +228,8 @@ __device__ __noinline__ void count_and_select(const VerifyParams& p, unsigned re
     __threadfence();
     const unsigned long long old = atomicAdd(&p.done[request], static_cast<unsigned long long>(n));
     // every element, and every row once for its draft logit
-    complete = old + n == static_cast<unsigned long long>(p.K + 1) * (static_cast<unsigned long long>(p.V) + 1) * p.nblk;
+    complete = old + n == static_cast<unsigned long long>(p.K + 1) *
+                              (static_cast<unsigned long long>(p.V) + 1) * p.nblk;
   }
   for (unsigned left = __ballot_sync(kFull, complete); left; left &= left - 1) {
     __threadfence();
@@ -334,7 +335,9 @@ __device__ __forceinline__ uint32_t first_cta_address(const void* smem) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(smem)));
   return r;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 struct SmallPlan {
@@ -408,10 +411,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     cluster_wait();  // the first CTA has started
     if (rank != 0 && warp == 0) {
       if (lane < K1)
-        asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(first_cta_address(&s_peer_key[rank][lane])), "l"(s_key[lane])
-                     : "memory");
+        asm volatile("st.shared::cluster.u64 [%0], %1;"
+                     ::"r"(first_cta_address(&s_peer_key[rank][lane])), "l"(s_key[lane]) : "memory");
       if (lane == 0)
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(first_cta_address(&s_peer_flags[rank])), "r"(s_flags) : "memory");
+        asm volatile("st.shared::cluster.u32 [%0], %1;"
+                     ::"r"(first_cta_address(&s_peer_flags[rank])), "r"(s_flags) : "memory");
       __syncwarp();
     }
     cluster_arrive();
@@ -1032,30 +1036,30 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
 //   kTma     resident inputs of at least kTmaMinBytes whose rows are at least
 //            kTmaMinRowBytes: a slice is streamed ahead of the kernels before
 //            it, which a unit's CTA, that has to wait for them when it ends,
-//            cannot (12.0 against 15.8 us per step of 87.5 MB with 304 KB rows).
-//            A slice pays for every row it enters: at 200 MB the two meet
-//            between 100 KB rows (35.6 against 31.7 us) and 128 KB rows (30.0
-//            against 31.1 us).
+//            cannot (11.7-12.1 against 14.5 us per step of 87.5 MB with 304 KB
+//            rows). A slice pays for every row it enters: with 100 KB rows it is
+//            10.6 against 11.3 us at 60 MB and 33.4 against 29.4 us at 200 MB,
+//            with 128 KB rows 10.2 against 11.2 and 29.3 both.
 //   kSmall   a request fits one round of loads of a cluster (508 KB; 60 KB for
 //            one CTA) and there are few enough: no hand-off to a selection, one
-//            launch. With one CTA each 2.4 against 3.0 us (8 requests of 18 KB),
-//            3.0 against 5.1 (152 of 18 KB), 4.8 against 6.0 us (128 of 54 KB).
-//            With a cluster 3.5 against 4.2 us (16 of 144 KB), no gain for one
-//            call alone that waits (3.25 us both, 2 of 320 KB) but half the
-//            launches, and 1.5 against 2.5 us with resident inputs. A GPU full of
-//            clusters of four or eight is slower: 7.2 against 5.7 us (19 of 504
-//            KB), 6.9 against 5.0 us (38 of 216 KB).
+//            launch. With one CTA each 2.5 against 3.0 us (8 requests of 18 KB),
+//            3.1 against 3.8 (152 of 18 KB), 4.9 against 5.0 us (128 of 54 KB);
+//            beyond a CTA per SM 5.4 against 4.6 us (256 of 18 KB). With a
+//            cluster 3.6 against 3.7 us (16 of 144 KB), 3.2 both (2 of 320 KB),
+//            but half the launches, and 1.5-1.7 against 2.4-2.7 us with resident
+//            inputs. A GPU full of clusters of four or eight is slower: 7.3
+//            against 5.1 us (19 of 504 KB), 7.0 against 5.0 us (38 of 216 KB).
 //   kStream  everything else. A call that waits for the kernel ahead of it has
-//            nothing to overlap and takes 15.5 us for 87.5 MB where the TMA
-//            pipeline took 20.5 us, 93 against 100 us for 662 MB, 4.0 against
-//            8.2 us for 2.7 MB, 7.0 against 26 us for 16 MB in 2 KB rows.
+//            nothing to overlap and takes 14.8-15.1 us for 87.5 MB where the TMA
+//            pipeline took 20.5 us, 91.7 against 100 us for 662 MB, 3.6 against
+//            8.2 us for 2.7 MB, 7 against 26 us for 16 MB in 2 KB rows.
 // The launch options can force a kernel (the tests use that to cover every
 // kernel); a forced `small` falls back to the default when the shape does not
 // qualify.
 constexpr long long kTmaMinBytes = 1LL << 20;
 constexpr long long kTmaMinRowBytes = 112LL << 10;
 constexpr long long kSmallMaxBytes = 1LL << 20;         // below this any number of one-CTA requests
-constexpr int kSmallMaxCtas = 304;                      // two a SM
+constexpr int kSmallMaxCtas = 152;                      // one a SM
 constexpr int kSmallMaxClusterCtas = 152;
 constexpr long long kSmallMaxClusterBytes = 5LL << 20;  // of clusters larger than two
 
@@ -1100,7 +1104,8 @@ StreamPlan stream_plan(const VerifyParams& p, long long rows, int sms) {
   long long per = ((rows * nvec + warps - 1) / warps + 31) / 32 * 32;
   per = per < 32 ? 32 : per > 32 * kStreamUnroll ? 32 * kStreamUnroll : per;
   q.per = static_cast<int>(per);
-  q.units = nvec <= per ? 1 : static_cast<int>((nvec + 7 + per - 1) / per);  // + 7: the first unit may begin inside a line
+  // + 7: the first unit may begin inside a line
+  q.units = nvec <= per ? 1 : static_cast<int>((nvec + 7 + per - 1) / per);
   q.line = first_line<T>(p);
   q.rows = static_cast<unsigned>(rows);
   q.by_units.set(static_cast<unsigned>(q.units));
@@ -1310,7 +1315,8 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches) {
   if (rc != ASD_OK) return rc;
   const long long request_bytes = static_cast<long long>(K + 1) * V * (dtype_code(dtype) == ASD_BF16 ? 2 : 4);
   const LaunchOptions opt = launch_options();
-  const Path path = choose_path(opt.path, request_bytes * B, request_bytes, B, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0);
+  const Path path =
+      choose_path(opt.path, request_bytes * B, request_bytes, B, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0);
   *launches = B == 0 ? 0 : (path != Path::kSmall && opt.split ? 2 : 1);
   return ASD_OK;
 }

@@ -1,8 +1,8 @@
-"""The row stages that cut rows into units, at the sizes where its cut of a row into units can go wrong: one vector
-either side of a unit, a unit of one, four and eight loads per lane, rows shorter than a vector, starts off the
-16-byte and the 128-byte grid, rows whose maximum sits at a unit's edge or is tied across units, rows of -inf,
-infinities and the lowest finite value; requests on both sides of each cluster size. Every output bit for bit the oracle's (comparisons and one fp32
-subtraction decide all of them)."""
+"""The row stages that cut rows into units, at the sizes where the cut can go wrong: one vector either side of
+a unit, a unit of one, four and eight loads per lane, rows shorter than a vector, starts off the 16-byte and the
+128-byte grid, rows whose maximum sits at a unit's edge or is tied across units, rows of -inf, infinities, the
+lowest finite value and subnormal maxima; requests on both sides of each cluster size; several blocks per call.
+Every output bit for bit the oracle's (comparisons and one fp32 subtraction decide all of them)."""
 import math
 
 import numpy as np
