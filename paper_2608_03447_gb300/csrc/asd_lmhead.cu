@@ -11,18 +11,19 @@
 // (tcgen05 cta_group::2). An MMA's M is 256 vocabulary rows (128 per SM: the
 // TMEM lanes), its N is one token tile (the TMEM columns): the T token rows are
 // cut into as few tiles of at most 256 columns as hold them, all of the same
-// width (T = 576: three of 192, no padding; T = 18: one of 32). A pair works
-// through items of two vocabulary tiles (512 rows) by one token tile: per
-// 64-deep K step each SM loads 2 x 128 rows of W and half of the token rows and
-// issues two MMAs per K slice over the same token slab, so the token rows cross
-// from L2 once per two vocabulary tiles. Items are dealt to the pairs in one
+// width (T = 576: three of 192, no padding; T = 18: one of 32). With several
+// token tiles a pair works through items of two vocabulary tiles (512 rows) by one
+// token tile: per 64-deep K step each SM loads 2 x 128 rows of W and half of the
+// token rows and issues two MMAs per K slice over the same token slab, so the token
+// rows cross from L2 once per two vocabulary tiles; with one token tile an item is
+// one vocabulary tile (see launch_lmhead). Items are dealt to the pairs in one
 // sequence, token tiles innermost, so the pairs that need a W row run at the
 // same time and it comes from HBM about once (see LmParams for the last round).
 // Per CTA: warp 0 issues TMA loads (128B-swizzled 64-wide K slabs) into a ring
 // of as many stages as fit, whose completion is counted on the first CTA's
 // barrier; warp 1 allocates tensor memory, and in the first CTA one of its
-// threads issues the MMAs; the other warps reduce the accumulators. Accumulators are
-// slots in a ring of two to four (512 columns / token tile width), each handed
+// threads issues the MMAs; the other warps reduce the accumulators. Accumulators
+// are slots in a ring of two to four (512 columns / token tile width), each handed
 // over by barriers of its own, so that the MMAs of the next item begin when one
 // tile has been read and run ahead in it while the other is being read.
 // The epilogue reads each 32 x 32 block (vocabulary rows x token columns) of a
@@ -51,19 +52,16 @@ constexpr int kHalfM = 128;               // vocabulary rows per CTA in one MMA 
 constexpr int kMaxTN = 256;               // most token rows per tile (MMA N; a multiple of 32)
 constexpr int kBK = 64;                   // K per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int kUmmaK = 16;                // K per tcgen05.mma (kind::f16)
-constexpr int kW = 2;                     // vocabulary tiles per item (MMAs per token slab)
-constexpr int kUnitM = kW * kPairM;       // vocabulary rows per item
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 12;
 constexpr int kSlabA = kHalfM * kBK * 2;  // 16 KB of vocabulary rows per tile
-constexpr int kStageA = kW * kSlabA;
 constexpr int kMaxSlots = 4;              // accumulators in tensor memory
 // Epilogue warps: a tile's 32-column blocks go in turn to the warps of each TMEM
 // lane quarter. A reduction that still has to look for its maxima (a pair's first
 // item) takes 1.2 us a block, and nothing hides it behind a pair's last item. With
 // one token tile, where that is what a call adds to streaming the weight, there are
-// sixteen warps instead of eight: 256 tokens on a 38912-row shard 73.5 us instead of
-// 77.2, 160 tokens 68.5 instead of 70.8, 18 tokens 65.3 instead of 65.7. With more
-// tiles (or logits to write) the tensor cores set the pace, and sixteen gain nothing.
+// sixteen warps instead of eight: on 38912 rows 73.5 us instead of 77.2 for 256
+// tokens, 68.5 instead of 70.8 for 160. With more tiles (or logits to write) the
+// tensor cores set the pace, and sixteen gain nothing.
 constexpr int kEpiWarpsOneTile = 16;
 constexpr int kEpiWarps = 8;
 constexpr int lm_threads(int epi_warps) { return (2 + epi_warps) * 32; }  // producer, MMA, epilogue warps
@@ -84,13 +82,16 @@ struct LmShared {
 };
 // dynamic shared memory: [1 KB alignment slack][stages x B][stages x A][LmShared]
 constexpr size_t kLmSmemMax = 232448;
-constexpr size_t lm_stage_bytes(int tn) { return kStageA + static_cast<size_t>(tn) / 2 * kBK * 2; }
-constexpr int lm_stages(int tn) {
-  const size_t fit = (kLmSmemMax - 1024 - sizeof(LmShared)) / lm_stage_bytes(tn);
-  return fit < kMaxStages ? static_cast<int>(fit) : kMaxStages;
+constexpr size_t lm_stage_bytes(int tn, int kw) { return kw * kSlabA + static_cast<size_t>(tn) / 2 * kBK * 2; }
+constexpr int lm_stages(int tn, int kw) {
+  const size_t fit = (kLmSmemMax - 1024 - sizeof(LmShared)) / lm_stage_bytes(tn, kw);
+  const int most = kw == 1 ? kMaxStages : kMaxStages / 2;
+  return fit < static_cast<size_t>(most) ? static_cast<int>(fit) : most;
 }
-constexpr size_t lm_smem_bytes(int tn) { return 1024 + lm_stages(tn) * lm_stage_bytes(tn) + sizeof(LmShared); }
-static_assert(lm_stages(192) == 5 && lm_stages(kMaxTN) == 4, "ring depth at the widths that serve most");
+constexpr size_t lm_smem_bytes(int tn, int kw) {
+  return 1024 + lm_stages(tn, kw) * lm_stage_bytes(tn, kw) + sizeof(LmShared);
+}
+static_assert(lm_stages(192, 2) == 5 && lm_stages(kMaxTN, 2) == 4, "ring depth at the widths that serve most");
 
 // ---------------------------------------------------------------- tcgen05 / TMA / cluster helpers
 
@@ -406,7 +407,7 @@ struct LmParams {
   int stages;       // ring stages
   int slots;        // accumulator slots
   int k_steps;      // ceil(H / kBK)
-  // Items 0 .. full - 1: item i is vocabulary rows (i / token_tiles) * kUnitM on by token tile i % token_tiles.
+  // Items 0 .. full - 1: item i is vocabulary rows (i / token_tiles) * kw * kPairM on by token tile i % token_tiles.
   // When the last round of the deal would leave more than half of the pairs idle, its items are dealt in
   // halves (one vocabulary tile each): entries full + 2 h and full + 2 h + 1 are the tiles of item full + h.
   int full, entries;
@@ -419,18 +420,20 @@ struct LmItem {
   int kw;    // vocabulary tiles
   int m;     // token tile
 };
+template <int kW>
 __device__ __forceinline__ LmItem lm_item(const LmParams& q, int entry) {
   const int half = entry - q.full;
   const int item = half < 0 ? entry : q.full + (half >> 1);
   LmItem it;
   it.m = item % q.token_tiles;
-  it.row0 = (item / q.token_tiles) * kUnitM + (half < 0 ? 0 : (half & 1) * kPairM);
-  it.kw = half < 0 && it.row0 + kPairM < q.V ? kW : 1;  // no second tile past the vocabulary
+  it.row0 = (item / q.token_tiles) * (kW * kPairM) + (half < 0 ? 0 : (half & 1) * kPairM);
+  it.kw = kW == 2 && half < 0 && it.row0 + kPairM < q.V ? 2 : 1;  // no second tile past the vocabulary
   return it;
 }
 
 // One CTA pair (cluster of 2) works through entries pair, pair + pairs, ...
-template <bool kWriteLogits, int kEpi>
+// kW: vocabulary tiles per item.
+template <bool kWriteLogits, int kEpi, int kW>
 __global__ void __launch_bounds__(lm_threads(kEpi), 1)
     lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w,
                          const __grid_constant__ VerifyParams p, const __grid_constant__ LmParams q) {
@@ -441,6 +444,7 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
   const int stages = q.stages;
   const uint32_t stage_b = static_cast<uint32_t>(q.tn) / 2 * kBK * 2;  // this CTA's half of the token rows
   const uint32_t sB = base;                                            // stages x stage_b
+  constexpr uint32_t kStageA = kW * kSlabA;
   const uint32_t sA = base + static_cast<uint32_t>(stages) * stage_b;  // stages x kStageA
   LmShared& sh = *reinterpret_cast<LmShared*>(gbase + static_cast<uint32_t>(stages) * (kStageA + stage_b));
 
@@ -499,7 +503,7 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
     uint32_t ph = 0;
     bool ok = true;
     for (int e = pair; ok && e < q.entries; e += pairs) {
-      const LmItem it = lm_item(q, e);
+      const LmItem it = lm_item<kW>(q, e);
       const int tok = it.m * q.tn + static_cast<int>(rank) * (q.tn / 2);
       const int row = it.row0 + static_cast<int>(rank) * kHalfM;
       const uint32_t tx = 2u * (static_cast<uint32_t>(it.kw) * kSlabA + stage_b);  // both CTAs' bytes
@@ -535,7 +539,7 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
       const uint64_t a_desc = smem_desc_sw128(sA), b_desc = smem_desc_sw128(sB);
       // the MMAs of one K step of vocabulary tile j: stage s into the accumulator at column d
       auto mma_step = [&](int s, int j, uint32_t d, bool first) {
-        const uint64_t ad = a_desc + static_cast<uint32_t>((s * kStageA + j * kSlabA) >> 4);
+        const uint64_t ad = a_desc + static_cast<uint32_t>((s * static_cast<int>(kStageA) + j * kSlabA) >> 4);
         const uint64_t bd = b_desc + ((static_cast<uint32_t>(s) * stage_b) >> 4);
 #pragma unroll
         for (int kk = 0; kk < kBK / kUmmaK; ++kk)  // 16 elements (32 bytes, encoded 2) along K inside the swizzle row
@@ -547,7 +551,7 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
       uint32_t slot_ph = 1;
       bool ok = true;
       for (int e = pair; ok && e < q.entries; e += pairs) {
-        const int kw = lm_item(q, e).kw;
+        const int kw = lm_item<kW>(q, e).kw;
         const int slot0 = slot;
         const uint32_t d0 = tmem + static_cast<uint32_t>(slot0 * q.tn);
         ok = mbar_wait_warp(&sh.acc_empty[slot0], slot_ph, &sh.abort);
@@ -617,13 +621,11 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
       __syncwarp();
     }
   } else {
-    // ---------------- epilogue: warps 2 on, each on one TMEM lane quarter. The warps of a quarter deal its
-    // 32-column blocks in turn; with four, the second tile's on from the first's, so that tiles of few blocks are
-    // read by different warps.
+    // ---------------- epilogue: warps 2 on, each on one TMEM lane quarter, whose warps take turns at the 32-column
+    // blocks of every accumulator
     constexpr int kTurns = kEpi / 4;
     const int quarter = warp & 3;  // TMEM lanes this warp may read
     const int turn = (warp - 2) >> 2;
-    const int blocks = q.tn / 32;
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const uint32_t acc_empty0 = map_rank(smem_u32(&sh.acc_empty[0]), 0);
     const int et = static_cast<int>(threadIdx.x) - 64;  // this thread among the epilogue's: its token column
@@ -631,7 +633,7 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
     uint32_t slot_ph = 0;
     bool ok = true;
     for (int e = pair; e < q.entries; e += pairs) {
-      const LmItem it = lm_item(q, e);
+      const LmItem it = lm_item<kW>(q, e);
       const int tok0 = it.m * q.tn;
       // While the item's MMAs run: its draft tokens, and what each token has to beat, over all CTAs so far
       const bool has_token = et < q.tn && tok0 + et < q.T;
@@ -667,8 +669,7 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
           const uint32_t acc = tmem + lane_base + static_cast<uint32_t>(slot * q.tn);
           const int v_warp = it.row0 + t * kPairM + static_cast<int>(rank) * kHalfM + quarter * 32;
           if (v_warp < q.V) {  // rows past the vocabulary: nothing to reduce
-            const int c_first = (kTurns == 4 ? (turn + t * (kTurns - blocks % kTurns)) % kTurns : turn) * 32;
-            for (int c = c_first; c < q.tn; c += kTurns * 32) {
+            for (int c = turn * 32; c < q.tn; c += kTurns * 32) {
               if (kWriteLogits) {
                 const int v = v_warp + lane;  // this thread's vocabulary row
                 uint32_t r[32];
@@ -768,7 +769,7 @@ struct LmDevice {
   int major = 0, minor = 0;
   // CTA pairs resident at once, per kernel instance (0: not set up yet); the
   // set-up is idempotent, so two threads racing to do it store the same value
-  std::atomic<int> pairs[3] = {};
+  std::atomic<int> pairs[4] = {};
 };
 
 int lm_device(LmDevice** out) {
@@ -818,32 +819,33 @@ cudaLaunchConfig_t pair_config(unsigned grid, int threads, size_t smem, cudaStre
 // The last round of the deal: `left` items for more pairs. Up to half of the
 // pairs' number, half items keep twice as many pairs busy for half the time;
 // beyond that, halves would only begin a second round.
-void lm_plan(int T, int V, int H, int pairs, LmParams* q) {
+void lm_plan(int T, int V, int H, int kw, int pairs, LmParams* q) {
   q->T = T;
   q->H = H;
   q->V = V;
   q->token_tiles = (T + kMaxTN - 1) / kMaxTN;
   const int per = (T + q->token_tiles - 1) / q->token_tiles;
   q->tn = (per + 31) / 32 * 32;
-  q->stages = lm_stages(q->tn);
+  q->stages = lm_stages(q->tn, kw);
   q->slots = kTmemCols / q->tn < kMaxSlots ? kTmemCols / q->tn : kMaxSlots;
   q->k_steps = (H + kBK - 1) / kBK;
-  const int items = (V + kUnitM - 1) / kUnitM * q->token_tiles;
+  const int unit = kw * kPairM;
+  const int items = (V + unit - 1) / unit * q->token_tiles;
   const int left = items % pairs;
-  const int halved = 2 * left <= pairs ? left : 0;
+  const int halved = kw == 2 && 2 * left <= pairs ? left : 0;
   q->full = items - halved;
   q->entries = items + halved;
 }
 
-template <bool kWriteLogits, int kEpi>
+template <bool kWriteLogits, int kEpi, int kW>
 int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
                          cudaStream_t stream) {
   LmDevice* dev = nullptr;
   int rc = lm_device(&dev);
   if (rc != ASD_OK) return rc;
   if (dev->major != 10) return ASD_ERR_DEVICE;  // tcgen05 needs a Blackwell (sm_10x) device
-  auto kernel = lmhead_verify_kernel<kWriteLogits, kEpi>;
-  std::atomic<int>& resident = dev->pairs[kWriteLogits ? 1 : kEpi == kEpiWarps ? 0 : 2];
+  auto kernel = lmhead_verify_kernel<kWriteLogits, kEpi, kW>;
+  std::atomic<int>& resident = dev->pairs[2 * (kW - 1) + (kWriteLogits ? 1 : 0)];
   cudaLaunchAttribute attr[2];
   int pairs = resident.load(std::memory_order_acquire);
   if (pairs == 0) {
@@ -857,23 +859,31 @@ int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, V
     resident.store(pairs, std::memory_order_release);
   }
   LmParams q;
-  lm_plan(T, p.V, H, pairs, &q);
+  lm_plan(T, p.V, H, kW, pairs, &q);
   q.logits_out = logits_out;
   CUtensorMap map_h, map_w;
   if (!make_map(&map_h, hidden, T, H, q.tn / 2) || !make_map(&map_w, weight, p.V, H, kHalfM)) return ASD_ERR_CUDA;
   const unsigned grid = 2u * static_cast<unsigned>(q.entries < pairs ? q.entries : pairs);
-  cudaLaunchConfig_t cfg = pair_config(grid, lm_threads(kEpi), lm_smem_bytes(q.tn), stream, attr, true);
+  cudaLaunchConfig_t cfg = pair_config(grid, lm_threads(kEpi), lm_smem_bytes(q.tn, kW), stream, attr, true);
   if (cudaLaunchKernelEx(&cfg, kernel, map_h, map_w, p, q) != cudaSuccess) return ASD_ERR_CUDA;
   if (kWriteLogits) return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
   return launch_select<float, false>(p, true, stream);
 }
 
+// With one token tile an item is one vocabulary tile and a stage half as long (the
+// ring twice as deep): the token rows are read from L2 once more, but the first of
+// two tiles is reduced while the second one's weight streams, instead of both at
+// the end. On 38912 vocabulary rows 18 tokens take 60.9 us instead of 63.5, 64 61.4
+// instead of 63.8, 160 63.4 instead of 66.1, 256 68.5 instead of 71.4 (their logits
+// 74.3 instead of 76.5); on four times as many rows 222.5 / 223 / 228 / 245.5 us
+// instead of 226.5 / 227 / 229 / 249.5. With several token tiles the tensor cores
+// set the pace, and two vocabulary tiles per token slab feed them with less.
 template <bool kWriteLogits>
 int launch_lmhead(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
                   cudaStream_t stream) {
-  if (!kWriteLogits && T <= kMaxTN)
-    return launch_lmhead_kernel<kWriteLogits, kEpiWarpsOneTile>(hidden, weight, H, T, p, logits_out, stream);
-  return launch_lmhead_kernel<kWriteLogits, kEpiWarps>(hidden, weight, H, T, p, logits_out, stream);
+  if (T > kMaxTN) return launch_lmhead_kernel<kWriteLogits, kEpiWarps, 2>(hidden, weight, H, T, p, logits_out, stream);
+  constexpr int kEpi = kWriteLogits ? kEpiWarps : kEpiWarpsOneTile;
+  return launch_lmhead_kernel<kWriteLogits, kEpi, 1>(hidden, weight, H, T, p, logits_out, stream);
 }
 
 int check_lm_inputs(const void* hidden, const void* weight, int H) {
