@@ -365,11 +365,10 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches);
  *   path          ASD_PATH_AUTO picks the row-stage kernel by size (one CTA or
  *                 one cluster of CTAs per request, selection included, for few
  *                 requests that fit it; the TMA pipeline for
- *                 ASD_RESIDENT_INPUTS of at least 1 MB in rows of at least
- *                 112 KB; the register-streaming kernel for
- *                 everything else); the others force one (a forced
- *                 ASD_PATH_SMALL falls back to AUTO where the shape does not
- *                 fit it).
+ *                 ASD_RESIDENT_INPUTS in long rows (few, or more than 21 MB);
+ *                 the register-streaming kernel for everything else); the
+ *                 others force one (a forced ASD_PATH_SMALL falls back to AUTO
+ *                 where the shape does not fit it).
  *   fused_select  1: the row stage runs the selection itself (the CTA that
  *                 completes a request selects it) instead of launching
  *                 select_kernel right behind it.

@@ -1033,13 +1033,17 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
 }
 
 // Which kernel streams the logits.
-//   kTma     resident inputs of at least kTmaMinBytes whose rows are at least
-//            kTmaMinRowBytes: a slice is streamed ahead of the kernels before
-//            it, which a unit's CTA, that has to wait for them when it ends,
-//            cannot (11.7-12.1 against 14.5 us per step of 87.5 MB with 304 KB
-//            rows). A slice pays for every row it enters: with 100 KB rows it is
-//            10.6 against 11.3 us at 60 MB and 33.4 against 29.4 us at 200 MB,
-//            with 128 KB rows 10.2 against 11.2 and 29.3 both.
+//   kTma     resident inputs of more than kTmaMinBytes with long rows: a slice is
+//            streamed ahead of the kernels before it, which a unit's CTA, that has
+//            to wait for them when it ends, cannot (11.7-12.1 against 14.5 us per
+//            step of 87.5 MB with 304 KB rows) once the units of one call fill the
+//            GPU. Below that the next call's units find room beside them (4.2
+//            against 5.2 us at 17.9 MB with 64 KB rows, 6.1 against 5.7 at 21.9 MB)
+//            unless the rows are few (20 of 517 KB: 3.5 against 3.0 us).
+//            A slice pays for every row it enters: with 64 KB rows 7.2 against 7.3
+//            us at 27.6 MB (432 rows) but 8.7 against 8.3 at 37.4 MB (585), with
+//            112 KB rows 13.4 against 13.9 at 80 MB and 19.7 against 19.2 at 120 MB,
+//            with 128 KB rows 29.3 both at 200 MB.
 //   kSmall   a request fits one round of loads of a cluster (508 KB; 60 KB for
 //            one CTA) and there are few enough: no hand-off to a selection, one
 //            launch. With one CTA each 2.5 against 3.0 us (8 requests of 18 KB),
@@ -1056,8 +1060,12 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
 // The launch options can force a kernel (the tests use that to cover every
 // kernel); a forced `small` falls back to the default when the shape does not
 // qualify.
-constexpr long long kTmaMinBytes = 1LL << 20;
-constexpr long long kTmaMinRowBytes = 112LL << 10;
+constexpr long long kTmaMinBytes = 41LL << 19;           // 21.5 MB
+constexpr long long kTmaMinBytesFewRows = 1LL << 20;     // up to kTmaFewRows
+constexpr long long kTmaFewRows = 64;
+constexpr long long kTmaMinRowBytes = 64LL << 10;        // up to kTmaManyRows
+constexpr long long kTmaMinRowBytesManyRows = 112LL << 10;
+constexpr long long kTmaManyRows = 3 * 152;              // about three a slice
 constexpr long long kSmallMaxBytes = 1LL << 20;         // below this any number of one-CTA requests
 constexpr int kSmallMaxCtas = 152;                      // one a SM
 constexpr int kSmallMaxClusterCtas = 152;
@@ -1082,7 +1090,11 @@ Path choose_path(int forced, long long bytes, long long request_bytes, int B, in
   if (ctas > 1 && static_cast<long long>(B) * ctas <= kSmallMaxClusterCtas &&
       (ctas == 2 || bytes <= kSmallMaxClusterBytes))
     return Path::kSmall;
-  return resident && bytes >= kTmaMinBytes && request_bytes / (K + 1) >= kTmaMinRowBytes ? Path::kTma : Path::kStream;
+  const long long row_bytes = request_bytes / (K + 1), rows = bytes / row_bytes;
+  if (resident && bytes >= (rows <= kTmaFewRows ? kTmaMinBytesFewRows : kTmaMinBytes) &&
+      row_bytes >= (rows <= kTmaManyRows ? kTmaMinRowBytes : kTmaMinRowBytesManyRows))
+    return Path::kTma;
+  return Path::kStream;
 }
 
 // The cut of a row into units: as large as a warp's loads in flight allow, but

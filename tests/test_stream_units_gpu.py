@@ -64,21 +64,23 @@ def test_unit_edges(asd, dtype, vectors, fused):
         assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
 
 
-@pytest.mark.parametrize("row_bytes", [112 * 1024 - 2, 112 * 1024])
+@pytest.mark.parametrize("row_kb, B", [(64, 21), (64, 22), (64, 113), (64, 152), (64, 153),
+                                       (112, 63), (112, 153)])
+@pytest.mark.parametrize("short", [0, 2])
 @pytest.mark.parametrize("resident", [False, True])
-def test_both_sides_of_the_dispatch(asd, row_bytes, resident):
-    """Rows on both sides of the line between the two kernels for resident inputs, and of the 1 MB line."""
-    V, K = row_bytes // 2, 2
-    for B in (3, 4):
-        z = torch.randn(B, K + 1, V, device="cuda").mul_(3.0).to(torch.bfloat16)
-        draft = z[:, :K].argmax(2).to(torch.int32).contiguous()
-        draft[:, 1] = torch.randint(0, V, (B,), dtype=torch.int32, device="cuda")
-        ledger = asd.make_ledger(B, 8.0)
-        torch.cuda.synchronize()
-        out = asd.verify(z, draft, ledger, math.inf, 2, resident=resident)
-        torch.cuda.synchronize()
-        want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), math.inf, 2)
-        _equal(out, want, f"V={V} B={B}")
+def test_both_sides_of_the_dispatch(asd, row_kb, B, short, resident):
+    """Rows, their number and their bytes on both sides of the lines between the two kernels for resident
+    inputs (64 KB up to 456 rows, else 112 KB; 1 MB up to 64 rows, else 21.5 MB)."""
+    V, K = (row_kb * 1024 - short) // 2, 2
+    z = torch.randn(B, K + 1, V, device="cuda").mul_(3.0).to(torch.bfloat16)
+    draft = z[:, :K].argmax(2).to(torch.int32).contiguous()
+    draft[:, 1] = torch.randint(0, V, (B,), dtype=torch.int32, device="cuda")
+    ledger = asd.make_ledger(B, 8.0)
+    torch.cuda.synchronize()
+    out = asd.verify(z, draft, ledger, math.inf, 2, resident=resident)
+    torch.cuda.synchronize()
+    want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), math.inf, 2)
+    _equal(out, want, f"V={V} B={B}")
 
 
 @pytest.mark.parametrize("resident", [False, True])
