@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
             known = __ldcg(&p.row_key[tok]);
             // the row of this weight that holds the draft token (a vocabulary shard starts at global index
             // v_offset), if any
-            if (j < p.K) x = __ldg(p.draft + static_cast<long long>(b) * p.K + j) - p.v_offset;
+            if (j < p.K) x = __ldcg(p.draft + static_cast<long long>(b) * p.K + j) - p.v_offset;
             if (x < 0 || x >= p.V) x = -1;
           }
           sh.draft[et] = x;
