@@ -29,6 +29,7 @@
 
 #include "asd.h"
 #include "asd_device.cuh"
+#include "asd_dispatch.h"
 #include "asd_select.cuh"
 
 namespace {
@@ -324,11 +325,6 @@ __global__ void __launch_bounds__(kThreads, kSplit ? kStreamMinBlocks : 1)
 // vectors in flight) and merge the row keys in shared memory, the other CTAs hand
 // theirs to the first one, and its warp 0 runs Alg. 1; lane j of that warp has
 // fetched row j's draft token and its logit meanwhile. The workspace is not touched.
-
-constexpr int kSmallThreads = 512;
-constexpr int kSmallUnroll = 8;
-constexpr long long kSmallCtaBytes = 16LL * kSmallThreads * kSmallUnroll;  // 64 KB: one round of loads
-constexpr int kSmallMaxCluster = 8;                                        // the largest portable cluster
 
 __device__ __forceinline__ uint32_t first_cta_address(const void* smem) {
   uint32_t r;
@@ -955,7 +951,7 @@ LaunchOptions launch_options() {
 
 // SM count of the current device, and the one-time dynamic shared memory
 // opt-in of the TMA kernels, cached per device.
-int device_info(int* dev_out, DeviceInfo** info_out) {
+int device_info(DeviceInfo** info_out) {
   constexpr int kMaxDevices = 64;
   static DeviceInfo info[kMaxDevices];
   static std::mutex mu;
@@ -968,24 +964,15 @@ int device_info(int* dev_out, DeviceInfo** info_out) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return ASD_ERR_CUDA;
     info[dev].sms = sms;
   }
-  *dev_out = dev;
   *info_out = &info[dev];
   return ASD_OK;
 }
 
 template <typename T, bool kStrict>
-int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
+int launch_tma(const VerifyParams& p, DeviceInfo* info, const LaunchOptions& opt, cudaStream_t stream) {
   constexpr int VN = Elem<T>::kVec;
   constexpr long long kMinPerCta = 2LL * kTmaChunkBytes / static_cast<long long>(sizeof(T));
-  const uintptr_t addr = reinterpret_cast<uintptr_t>(p.logits);
-  if (addr % sizeof(T) != 0) return ASD_ERR_ALIGN;
-  long long head = static_cast<long long>(((16 - addr % 16) % 16) / sizeof(T));
-  if (head > p.total) head = p.total;
-  const long long bulk = (p.total - head) / VN * VN;
-  int dev = 0;
-  DeviceInfo* info = nullptr;
-  int rc = device_info(&dev, &info);
-  if (rc != ASD_OK) return rc;
+  const long long bulk = (p.total - p.head) / VN * VN;
   const bool split = opt.split;
   const int slot = (sizeof(T) == 2 ? 2 : 0) + (kStrict ? 1 : 0) + (split ? 4 : 0);
   if (!info->tma_ready[slot].load(std::memory_order_acquire)) {
@@ -1008,7 +995,6 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
   per_cta = (per_cta + VN - 1) / VN * VN;
   if (per_cta < VN) per_cta = VN;
   ncta = bulk > 0 ? (bulk + per_cta - 1) / per_cta : 1;
-  p.head = head;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(ncta));
   cfg.blockDim = dim3(kTmaThreads);
@@ -1021,7 +1007,7 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
   }
-  const long long bulk_end = head + bulk;
+  const long long bulk_end = p.head + bulk;
   if (!split) {
     if (cudaLaunchKernelEx(&cfg, verify_tma_kernel<T, kStrict, false>, p, bulk_end, per_cta) != cudaSuccess)
       return ASD_ERR_CUDA;
@@ -1030,71 +1016,6 @@ int launch_tma(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
   if (cudaLaunchKernelEx(&cfg, verify_tma_kernel<T, kStrict, true>, p, bulk_end, per_cta) != cudaSuccess)
     return ASD_ERR_CUDA;
   return launch_select<T, kStrict>(p, opt.pdl, stream);
-}
-
-// Which kernel streams the logits.
-//   kTma     resident inputs of more than kTmaMinBytes with long rows: a slice is
-//            streamed ahead of the kernels before it, which a unit's CTA, that has
-//            to wait for them when it ends, cannot (11.7-12.1 against 14.5 us per
-//            step of 87.5 MB with 304 KB rows) once the units of one call fill the
-//            GPU. Below that the next call's units find room beside them (4.2
-//            against 5.2 us at 17.9 MB with 64 KB rows, 6.1 against 5.7 at 21.9 MB)
-//            unless the rows are few (20 of 517 KB: 3.5 against 3.0 us).
-//            A slice pays for every row it enters: with 64 KB rows 7.2 against 7.3
-//            us at 27.6 MB (432 rows) but 8.7 against 8.3 at 37.4 MB (585), with
-//            112 KB rows 13.4 against 13.9 at 80 MB and 19.7 against 19.2 at 120 MB,
-//            with 128 KB rows 29.3 both at 200 MB.
-//   kSmall   a request fits one round of loads of a cluster (508 KB; 60 KB for
-//            one CTA) and there are few enough: no hand-off to a selection, one
-//            launch. With one CTA each 2.5 against 3.0 us (8 requests of 18 KB),
-//            3.1 against 3.8 (152 of 18 KB), 4.9 against 5.0 us (128 of 54 KB);
-//            beyond a CTA per SM 5.4 against 4.6 us (256 of 18 KB). With a
-//            cluster 3.6 against 3.7 us (16 of 144 KB), 3.2 both (2 of 320 KB),
-//            but half the launches, and 1.5-1.7 against 2.4-2.7 us with resident
-//            inputs. A GPU full of clusters of four or eight is slower: 7.3
-//            against 5.1 us (19 of 504 KB), 7.0 against 5.0 us (38 of 216 KB).
-//   kStream  everything else. A call that waits for the kernel ahead of it has
-//            nothing to overlap and takes 14.8-15.1 us for 87.5 MB where the TMA
-//            pipeline took 20.5 us, 91.7 against 100 us for 662 MB, 3.6 against
-//            8.2 us for 2.7 MB, 7 against 26 us for 16 MB in 2 KB rows.
-// The launch options can force a kernel (the tests use that to cover every
-// kernel); a forced `small` falls back to the default when the shape does not
-// qualify.
-constexpr long long kTmaMinBytes = 41LL << 19;           // 21.5 MB
-constexpr long long kTmaMinBytesFewRows = 1LL << 20;     // up to kTmaFewRows
-constexpr long long kTmaFewRows = 64;
-constexpr long long kTmaMinRowBytes = 64LL << 10;        // up to kTmaManyRows
-constexpr long long kTmaMinRowBytesManyRows = 112LL << 10;
-constexpr long long kTmaManyRows = 3 * 152;              // about three a slice
-constexpr long long kSmallMaxBytes = 1LL << 20;         // below this any number of one-CTA requests
-constexpr int kSmallMaxCtas = 152;                      // one a SM
-constexpr int kSmallMaxClusterCtas = 152;
-constexpr long long kSmallMaxClusterBytes = 5LL << 20;  // of clusters larger than two
-
-enum class Path { kSmall, kStream, kTma };
-
-// CTAs that take one request together: every lane's share in one round of loads
-// (0: too large).
-int small_cluster(long long request_bytes) {
-  for (int ctas = 1; ctas <= kSmallMaxCluster; ctas *= 2)
-    if (request_bytes <= ctas * kSmallCtaBytes - kSmallCtaBytes / (kSmallThreads / 32)) return ctas;
-  return 0;
-}
-
-Path choose_path(int forced, long long bytes, long long request_bytes, int B, int K, bool single_block, bool resident) {
-  const int ctas = single_block ? small_cluster(request_bytes) : 0;
-  if (forced == ASD_PATH_TMA) return Path::kTma;
-  if (forced == ASD_PATH_STREAM) return Path::kStream;
-  if (forced == ASD_PATH_SMALL && ctas > 0) return Path::kSmall;
-  if (ctas == 1 && (bytes < kSmallMaxBytes || B <= kSmallMaxCtas)) return Path::kSmall;
-  if (ctas > 1 && static_cast<long long>(B) * ctas <= kSmallMaxClusterCtas &&
-      (ctas == 2 || bytes <= kSmallMaxClusterBytes))
-    return Path::kSmall;
-  const long long row_bytes = request_bytes / (K + 1), rows = bytes / row_bytes;
-  if (resident && bytes >= (rows <= kTmaFewRows ? kTmaMinBytesFewRows : kTmaMinBytes) &&
-      row_bytes >= (rows <= kTmaManyRows ? kTmaMinRowBytes : kTmaMinRowBytesManyRows))
-    return Path::kTma;
-  return Path::kStream;
 }
 
 // The cut of a row into units: as large as a warp's loads in flight allow, but
@@ -1126,14 +1047,10 @@ StreamPlan stream_plan(const VerifyParams& p, long long rows, int sms) {
 }
 
 template <typename T, bool kStrict, bool kSplit>
-int launch_stream(VerifyParams& p, const LaunchOptions& opt, cudaStream_t stream) {
-  int dev = 0;
-  DeviceInfo* info = nullptr;
-  const int rc = device_info(&dev, &info);
-  if (rc != ASD_OK) return rc;
+int launch_stream(const VerifyParams& p, DeviceInfo* info, const LaunchOptions& opt, cudaStream_t stream) {
   const long long rows = static_cast<long long>(p.nblk) * p.B * (p.K + 1);
   StreamPlan q = stream_plan<T>(p, rows, info->sms);
-  if (rows >= kStreamMaxUnits / q.units) return launch_tma<T, kStrict>(p, opt, stream);
+  if (rows >= kStreamMaxUnits / q.units) return launch_tma<T, kStrict>(p, info, opt, stream);
   q.total = static_cast<unsigned>(rows * q.units);
   q.draft_ctas = p.K > 0 || !kSplit ? static_cast<unsigned>((rows + kThreads - 1) / kThreads) : 0;
   cudaLaunchConfig_t cfg = {};
@@ -1187,21 +1104,21 @@ int launch_small(const VerifyParams& p, int ctas, const LaunchOptions& opt, cuda
 
 template <typename T, bool kStrict>
 int launch(VerifyParams& p, cudaStream_t stream) {
+  const uintptr_t addr = reinterpret_cast<uintptr_t>(p.logits);
+  if (addr % sizeof(T) != 0) return ASD_ERR_ALIGN;
+  DeviceInfo* info = nullptr;
+  const int rc = device_info(&info);
+  if (rc != ASD_OK) return rc;
   const long long request_bytes = static_cast<long long>(p.K + 1) * p.V * static_cast<long long>(sizeof(T));
   const LaunchOptions opt = launch_options();
   const Path path = choose_path(opt.path, p.total * static_cast<long long>(sizeof(T)), request_bytes, p.B, p.K,
-                                p.nblk == 1 && !p.partials, p.resident != 0);
-  if (path == Path::kTma) return launch_tma<T, kStrict>(p, opt, stream);
-  const uintptr_t addr = reinterpret_cast<uintptr_t>(p.logits);
-  if (addr % sizeof(T) != 0) return ASD_ERR_ALIGN;
-  long long head = static_cast<long long>(((16 - addr % 16) % 16) / sizeof(T));
-  if (head > p.total) head = p.total;
-  if (path == Path::kSmall) {
-    p.head = head;
-    return launch_small<T, kStrict>(p, small_cluster(request_bytes), opt, stream);
-  }
-  p.head = head;
-  return opt.split ? launch_stream<T, kStrict, true>(p, opt, stream) : launch_stream<T, kStrict, false>(p, opt, stream);
+                                p.nblk == 1 && !p.partials, p.resident != 0, info->sms);
+  const long long head = static_cast<long long>(((16 - addr % 16) % 16) / sizeof(T));
+  p.head = head < p.total ? head : p.total;
+  if (path == Path::kTma) return launch_tma<T, kStrict>(p, info, opt, stream);
+  if (path == Path::kSmall) return launch_small<T, kStrict>(p, small_cluster(request_bytes), opt, stream);
+  return opt.split ? launch_stream<T, kStrict, true>(p, info, opt, stream)
+                   : launch_stream<T, kStrict, false>(p, info, opt, stream);
 }
 
 int verify_common(bool strict, const void* logits, int dtype, int B, int K, int V,
@@ -1327,8 +1244,14 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches) {
   if (rc != ASD_OK) return rc;
   const long long request_bytes = static_cast<long long>(K + 1) * V * (dtype_code(dtype) == ASD_BF16 ? 2 : 4);
   const LaunchOptions opt = launch_options();
+  DeviceInfo* info = nullptr;
+  int sms = kMeasuredSms;  // where there is no device to ask
+  if (device_info(&info) == ASD_OK)
+    sms = info->sms;
+  else
+    cudaGetLastError();  // not the caller's
   const Path path =
-      choose_path(opt.path, request_bytes * B, request_bytes, B, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0);
+      choose_path(opt.path, request_bytes * B, request_bytes, B, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0, sms);
   *launches = B == 0 ? 0 : (path != Path::kSmall && opt.split ? 2 : 1);
   return ASD_OK;
 }
