@@ -39,7 +39,11 @@ constexpr int kMeasuredSms = 152;
 //            one CTA) and there are few enough: no hand-off to a selection, one
 //            launch. With one CTA each 2.5 against 3.0 us (8 requests of 18 KB),
 //            3.1 against 3.8 (152 of 18 KB), 4.9 against 5.0 us (128 of 54 KB);
-//            beyond a CTA per SM 5.4 against 4.6 us (256 of 18 KB). With a
+//            beyond a CTA per SM 5.4 against 4.6 us (256 of 18 KB). A request of few
+//            and short rows has a CTA of few warps (small_plan); below a megabyte as
+//            many as fit the SMs at once: 3.2 against 3.9 us (1024 of 34 bytes), 3.2
+//            against 4.0 (304 of 1.8 KB), but 5.4 against 4.4 us (400 of 1.8 KB, two
+//            at a time on an SM) and 6.5 against 4.6 (4096 of 4 bytes). With a
 //            cluster 3.6 against 3.7 us (16 of 144 KB), 3.2 both (2 of 320 KB),
 //            but half the launches, and 1.5-1.7 against 2.4-2.7 us with resident
 //            inputs. A GPU full of clusters of four or eight is slower: 7.3
@@ -57,7 +61,8 @@ constexpr long long kTmaFewRows = 64;
 constexpr long long kTmaMinRowBytes = 64LL << 10;        // up to kTmaManyRows
 constexpr long long kTmaMinRowBytesManyRows = 112LL << 10;
 constexpr long long kTmaManyRows = 3;                    // a slice, of which there is one a SM
-constexpr long long kSmallMaxBytes = 1LL << 20;         // below this any number of one-CTA requests
+constexpr long long kSmallMaxBytes = 1LL << 20;         // below this as many one-CTA requests as fit at once
+constexpr int kSmallWarpsPerSm = 22;                    // at 88 registers a thread
 constexpr long long kSmallMaxClusterBytes = 5LL << 20;  // of clusters larger than two
 
 enum class Path { kSmall, kStream, kTma };
@@ -70,13 +75,40 @@ inline int small_cluster(long long request_bytes) {
   return 0;
 }
 
+// How verify_small_kernel cuts a request: every row into `units`, cut every `per`
+// vectors (a multiple of 32), for the CTAs' warps, one of which fetches the drafts'
+// logits instead. A request's only CTA has no more warps than units: sixteen for
+// every request let one CTA onto an SM at a time, and 256 requests of 34 bytes took
+// 4.6 us instead of 2.7, 1024 of them 14.5 us instead of 3.2.
+struct SmallPlan {
+  int units;
+  int per;
+  int warps;  // per CTA
+  int line;   // where in its 128-byte line the first vector of the logits lies
+};
+// nvec: whole vectors of a row, at most.
+inline SmallPlan small_plan(int nvec, int K, int ctas) {
+  SmallPlan q = {};
+  q.warps = kSmallThreads / 32;
+  const int warps = ctas * q.warps - 1;
+  const int share = warps / (K + 1) > 0 ? warps / (K + 1) : 1;  // units of a row that start at once
+  q.per = ((nvec + 7 + share - 1) / share + 31) / 32 * 32;
+  if (q.per > 32 * kSmallUnroll) q.per = 32 * kSmallUnroll;
+  q.units = nvec <= q.per ? 1 : (nvec + 7 + q.per - 1) / q.per;  // + 7: the first unit may begin inside a line
+  if (ctas == 1 && (K + 1) * q.units + 1 < q.warps) q.warps = (K + 1) * q.units + 1;
+  return q;
+}
+
 inline Path choose_path(int forced, long long bytes, long long request_bytes, int B, int K, bool single_block,
                         bool resident, int sms) {
   const int ctas = single_block ? small_cluster(request_bytes) : 0;
   if (forced == ASD_PATH_TMA) return Path::kTma;
   if (forced == ASD_PATH_STREAM) return Path::kStream;
   if (forced == ASD_PATH_SMALL && ctas > 0) return Path::kSmall;
-  if (ctas == 1 && (bytes < kSmallMaxBytes || B <= sms)) return Path::kSmall;
+  if (ctas == 1) {
+    const int warps = small_plan(static_cast<int>(request_bytes / (K + 1) / 16), K, 1).warps;
+    if (B <= (bytes < kSmallMaxBytes ? kSmallWarpsPerSm / warps : 1) * static_cast<long long>(sms)) return Path::kSmall;
+  }
   if (ctas > 1 && static_cast<long long>(B) * ctas <= sms &&
       (ctas == 2 || bytes <= kSmallMaxClusterBytes))
     return Path::kSmall;

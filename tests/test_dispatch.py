@@ -40,6 +40,14 @@ def test_one_cta_requests_of_a_megabyte_up_to_a_cta_per_sm(path_of, sms):
 
 
 @pytest.mark.parametrize("sms", [152, 76])
+@pytest.mark.parametrize("K,row,per_sm", [(0, 34, 11), (4, 200, 3), (8, 200, 2), (31, 8, 1), (0, 1000, 5), (14, 4, 1)])
+def test_tiny_requests_as_many_as_fit_at_once(path_of, K, row, per_sm, sms):
+    """A CTA of one warp per unit and one for the drafts' logits; 22 warps fit an SM."""
+    assert path_of(per_sm * sms, K, row, sms=sms) == SMALL
+    assert path_of(per_sm * sms + 1, K, row, sms=sms) == STREAM
+
+
+@pytest.mark.parametrize("sms", [152, 76])
 def test_clusters_of_two_up_to_a_cta_per_sm(path_of, sms):
     row = 20 * KB  # four rows: 80 KB a request
     assert path_of(sms // 2, 3, row, sms=sms) == SMALL

@@ -121,6 +121,39 @@ def test_request_clusters(asd, ctas, K, resident):
             assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
 
 
+@pytest.mark.parametrize("resident", [False, True])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("K,V,B", [(0, 1, 1672), (0, 17, 1673), (1, 9, 1064), (4, 100, 456), (4, 100, 457),
+                                   (8, 255, 304), (8, 257, 305), (13, 5, 152), (14, 5, 152), (15, 5, 153),
+                                   (31, 2, 152), (31, 33, 153), (0, 263, 200), (0, 520, 200), (2, 1100, 150)])
+def test_tiny_requests(asd, K, V, B, dtype, resident):
+    """Requests whose CTA has two to sixteen warps, with units of a load per lane and of more, as many as fit the
+    GPU at once and one more; tied tops, a top at either end of a row, a NaN in one request."""
+    vn = VEC[dtype]
+    off = (V + B) % vn
+    flat = torch.randn(off + B * (K + 1) * V, device="cuda").mul_(3.0).to(dtype)
+    z = flat[off:].view(B, K + 1, V)
+    z[0, :, 0] = 40.0
+    z[1, :, V - 1] = 40.0
+    z[2, :, V // 2:] = 40.0
+    z[3] = -math.inf
+    z[4, K, V // 3] = math.nan
+    draft = torch.randint(0, V, (B, K), dtype=torch.int32, device="cuda")
+    half = (K + 1) // 2
+    draft[:, :half] = z[:, :half].float().nan_to_num(0.0, 9e9, -9e9).argmax(2).to(torch.int32)
+    ledger = asd.make_ledger(B, 8.0)
+    torch.cuda.synchronize()
+    out = asd.verify(z, draft, ledger, 1.0, 2, resident=resident)
+    torch.cuda.synchronize()
+    want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), 1.0, 2)
+    assert np.array_equal(out["status"].cpu().numpy(), want["status"])
+    clean = want["status"] == 0
+    assert clean.sum() == B - 1
+    got = {k: v[torch.from_numpy(clean).cuda()] for k, v in out.items()}
+    _equal(got, {k: v[clean] for k, v in want.items() if k != "ledger"}, f"K={K} V={V} B={B} {dtype}")
+    assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
+
+
 @pytest.mark.parametrize("nblk", [2, 7, 8, 9, 17])
 def test_blocks_around_the_warps_of_a_selection(asd, nblk):
     """The ledger goes through fewer, as many and more blocks than the selection's CTA has warps; one block in
