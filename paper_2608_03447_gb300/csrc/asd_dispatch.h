@@ -45,9 +45,16 @@ constexpr int kMeasuredSms = 152;
 //            against 4.0 (304 of 1.8 KB), but 5.4 against 4.4 us (400 of 1.8 KB, two
 //            at a time on an SM) and 6.5 against 4.6 (4096 of 4 bytes). With a
 //            cluster 3.6 against 3.7 us (16 of 144 KB), 3.2 both (2 of 320 KB),
-//            but half the launches, and 1.5-1.7 against 2.4-2.7 us with resident
-//            inputs. A GPU full of clusters of four or eight is slower: 7.3
-//            against 5.1 us (19 of 504 KB), 7.0 against 5.0 us (38 of 216 KB).
+//            and with resident inputs 1.5-1.7 against 2.4-2.7 us; half the launches,
+//            which is what an eager call waits for (6.5 against 8.7 us). A GPU full
+//            of clusters is slower: of two CTAs 2.6 against 2.8 us at 60 of 72 KB
+//            but 3.4 against 2.9 at 76 (resident; 3.8 against 3.7 waiting), of four
+//            2.8 both at 32 of 130 KB but 3.3 against 2.8 at 36, of eight 3.1 both
+//            at 14 of 261 KB but 4.1 against 3.1 at 16, where they are no longer
+//            resident at once. The line for all is a CTA per SM, for the launch
+//            saved, up to 5 MB of clusters of four and eight (2.8 both at 14 of 360
+//            KB, 5.0 MB, 4.4 against 2.8 at 16, 5.8 MB); with resident inputs, which
+//            come in captured rounds, no more clusters of eight than fit at once.
 //   kStream  everything else. A call that waits for the kernel ahead of it has
 //            nothing to overlap and takes 14.8-15.1 us for 87.5 MB where the TMA
 //            pipeline took 20.5 us, 91.7 against 100 us for 662 MB, 3.6 against
@@ -64,6 +71,7 @@ constexpr long long kTmaManyRows = 3;                    // a slice, of which th
 constexpr long long kSmallMaxBytes = 1LL << 20;         // below this as many one-CTA requests as fit at once
 constexpr int kSmallWarpsPerSm = 22;                    // at 88 registers a thread
 constexpr long long kSmallMaxClusterBytes = 5LL << 20;  // of clusters larger than two
+constexpr int kSmallMaxLargestClusters = 14;            // resident inputs: at once on kMeasuredSms
 
 enum class Path { kSmall, kStream, kTma };
 
@@ -109,8 +117,8 @@ inline Path choose_path(int forced, long long bytes, long long request_bytes, in
     const int warps = small_plan(static_cast<int>(request_bytes / (K + 1) / 16), K, 1).warps;
     if (B <= (bytes < kSmallMaxBytes ? kSmallWarpsPerSm / warps : 1) * static_cast<long long>(sms)) return Path::kSmall;
   }
-  if (ctas > 1 && static_cast<long long>(B) * ctas <= sms &&
-      (ctas == 2 || bytes <= kSmallMaxClusterBytes))
+  if (ctas > 1 && static_cast<long long>(B) * ctas <= sms && (ctas == 2 || bytes <= kSmallMaxClusterBytes) &&
+      !(resident && ctas == kSmallMaxCluster && B > kSmallMaxLargestClusters * sms / kMeasuredSms))
     return Path::kSmall;
   const long long row_bytes = request_bytes / (K + 1), rows = bytes / row_bytes;
   if (resident && bytes >= (rows <= kTmaFewRows ? kTmaMinBytesFewRows : kTmaMinBytes * sms / kMeasuredSms) &&

@@ -48,10 +48,21 @@ def test_tiny_requests_as_many_as_fit_at_once(path_of, K, row, per_sm, sms):
 
 
 @pytest.mark.parametrize("sms", [152, 76])
-def test_clusters_of_two_up_to_a_cta_per_sm(path_of, sms):
-    row = 20 * KB  # four rows: 80 KB a request
-    assert path_of(sms // 2, 3, row, sms=sms) == SMALL
-    assert path_of(sms // 2 + 1, 3, row, sms=sms) == STREAM
+@pytest.mark.parametrize("resident", [False, True])
+def test_clusters_up_to_a_cta_per_sm(path_of, sms, resident):
+    """And with resident inputs no more clusters of eight than are resident at once."""
+    for ctas, row in ((2, 20 * KB), (4, 33 * KB), (8, 65 * KB)):
+        most = (14 * sms // 152) if resident and ctas == 8 else sms // ctas
+        assert path_of(most, 3, row, resident=resident, sms=sms) == SMALL
+        assert path_of(most + 1, 3, row, resident=resident, sms=sms) != SMALL
+
+
+def test_clusters_of_four_and_eight_up_to_five_megabytes(path_of):
+    assert path_of(76, 3, 30 * KB) == SMALL                       # clusters of two: 9 MB
+    assert path_of(20, 3, 62 * KB) == SMALL                       # of four
+    assert path_of(21, 3, 62 * KB) == STREAM
+    assert path_of(10, 3, 127 * KB - 16) == SMALL                 # of eight
+    assert path_of(11, 3, 127 * KB - 16) == STREAM
 
 
 @pytest.mark.parametrize("sms", [152, 76])
