@@ -20,15 +20,22 @@ using namespace asd_detail;
 
 constexpr int kCombineThreads = 256;
 // Shards whose partials are in flight at once, beside the ledger and the draft:
-// read shard by shard the combine was five L2 round trips in a row (a captured
-// partials + combine pair at B=32, K=8 over a 37984-entry shard of four:
-// 8.9 -> 8.5 us; at B=1: 5.2 -> 4.8 us).
+// read shard by shard the combine was five L2 round trips in a row.
 constexpr int kCombineBatch = 4;
 
-// Past L1: with programmatic dependent launch a line of it may be older than the kernel ahead.
+// Through L1, since the three words of a partial share their sectors with the
+// neighbouring lanes' (griddepcontrol.wait makes the writes of the kernels ahead
+// visible to ordinary loads; not left to the compiler, which may choose the read-only
+// path for a pointer that the kernel does not write through). Past L1 each word asked
+// for its sector again: 8 shards of 32 requests took 2.58 us where shard by shard it
+// had been 2.46, and 16 of 5000 requests of 32 rows 16.4 where it had been 8.0 (now
+// 2.37 and 7.2). Four shards of 32 requests: 2.19 shard by shard, 1.88, now 1.76 us.
 __device__ __forceinline__ asd_partial load_partial(const asd_partial* at) {
   const unsigned long long* w = reinterpret_cast<const unsigned long long*>(at);
-  const unsigned long long key = __ldcg(w), values = __ldcg(w + 1), flags = __ldcg(w + 2);
+  unsigned long long key, values, flags;
+  asm volatile("ld.global.u64 %0, [%1];" : "=l"(key) : "l"(w));
+  asm volatile("ld.global.u64 %0, [%1];" : "=l"(values) : "l"(w + 1));
+  asm volatile("ld.global.u64 %0, [%1];" : "=l"(flags) : "l"(w + 2));
   asd_partial q;
   q.key = key;
   q.top = __uint_as_float(static_cast<uint32_t>(values));
@@ -68,8 +75,12 @@ __global__ void __launch_bounds__(kCombineThreads) shard_combine_kernel(const as
       for (int s0 = 1; s0 < S; s0 += kCombineBatch) {
         asd_partial q[kCombineBatch];
 #pragma unroll
-        for (int i = 0; i < kCombineBatch; ++i)  // past the last shard: that shard again, which changes nothing
-          q[i] = load_partial(parts + static_cast<long long>(min(s0 + i, S - 1)) * R + row);
+        for (int i = 0; i < kCombineBatch; ++i) {
+          q[i].key = 0ull;  // past the last shard: what changes nothing
+          q[i].draft_logit = -INFINITY;
+          q[i].flags = 0u;
+          if (s0 + i < S) q[i] = load_partial(parts + static_cast<long long>(s0 + i) * R + row);
+        }
 #pragma unroll
         for (int i = 0; i < kCombineBatch; ++i) {
           if (q[i].key > best.key) best = q[i];

@@ -99,3 +99,20 @@ def test_shard_arguments_are_checked(asd):
     blk = inputs.gen_block(2, 2, 100, torch.float32, 3, "cuda")
     with pytest.raises(asd.AsdError):
         asd.shard_partials(blk.logits, blk.draft, 50, 120)  # shard past the end of the vocabulary
+
+
+@pytest.mark.parametrize("shards", [1, 2, 4, 5, 6, 8, 9, 13, 17])
+@pytest.mark.parametrize("B,K", [(1, 31), (9, 4), (300, 1)])
+def test_any_number_of_shards(asd, shards, B, K):
+    """Fewer, as many and more shards than the combine loads at once, on its edges."""
+    V = 1700
+    blk = inputs.gen_block(B, K, V, torch.bfloat16, 21_000 + shards, "cuda")
+    bounds = np.linspace(0, V, shards + 1).astype(int).tolist()
+    ledger = asd.make_ledger(B, 4.0)
+    out = run_sharded(asd, blk.logits, blk.draft, bounds, ledger, 1.0, 2)
+    torch.cuda.synchronize()
+    o = oracle.verify(blk.logits.cpu(), blk.draft.cpu().numpy(), np.array([[4.0, 0.0]] * B, np.float32), 1.0, 2)
+    for key in ("accepted_len", "committed", "recovery", "row_argmax", "status"):
+        assert np.array_equal(out[key].cpu().numpy(), o[key]), key
+    assert np.array_equal(out["row_regret"].cpu().numpy().view(np.uint32), o["row_regret"].view(np.uint32))
+    assert np.array_equal(ledger.cpu().numpy().view(np.uint32), o["ledger"].view(np.uint32))
