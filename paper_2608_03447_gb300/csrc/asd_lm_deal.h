@@ -1,0 +1,57 @@
+// How the fused LM head cuts token and vocabulary rows into items and deals them
+// to the CTA pairs: plain host arithmetic.
+#pragma once
+
+namespace asd_detail {
+
+constexpr int kPairM = 256;  // vocabulary rows per CTA pair in one MMA (MMA M)
+constexpr int kMaxTN = 256;  // most token rows per tile (MMA N; a multiple of 32)
+
+struct LmDeal {
+  int tn;           // token rows per tile
+  int token_tiles;  // ceil(T / tn)
+  // Items 0 .. full - 1: item i is vocabulary rows (i / token_tiles) * kw * kPairM on by token tile i % token_tiles.
+  // When the last round of the deal would leave more than half of the pairs idle, its items are dealt in
+  // halves (one vocabulary tile each): entries full + 2 h and full + 2 h + 1 are the tiles of item full + h.
+  int full, entries;
+};
+
+// Vocabulary units of kw tiles.
+inline int lm_units(int V, int kw) { return 1 + (V - 1) / (kw * kPairM); }
+
+// The most token rows of one launch: the kernel counts items in 32 bits, and the
+// largest vocabularies and batches have more (V = 2^31 - 1 with 2^17 rows: 2^31).
+// A call with more rows takes several launches, of at least 65536 rows each.
+#ifndef ASD_LM_MAX_ITEMS
+#define ASD_LM_MAX_ITEMS (1 << 30)  // tests of the split lower it
+#endif
+inline int lm_rows_per_launch(int V) {
+  const int tiles = ASD_LM_MAX_ITEMS / lm_units(V, 2);
+  return (tiles > 1 ? tiles < (1 << 22) ? tiles : 1 << 22 : 1) * kMaxTN;
+}
+
+// How T token rows and V vocabulary rows are cut and dealt to `pairs` CTA pairs.
+//
+// Token tiles: as few as hold T at up to 256 columns (each tile reads W once
+// more from L2, and a wider MMA reads its vocabulary operand from shared memory
+// less often per product), all of one width, rounded up to the 32 columns of an
+// epilogue block. Against a fixed width of 192: 320 rows took 384 columns and
+// take 2 x 160, 18 rows take 32, 2304 rows take 9 tiles instead of 12.
+//
+// The last round of the deal: `left` items for more pairs. Up to half of the
+// pairs' number, half items keep twice as many pairs busy for half the time;
+// beyond that, halves would only begin a second round.
+inline LmDeal lm_deal(int T, int V, int kw, int pairs) {
+  LmDeal d;
+  d.token_tiles = 1 + (T - 1) / kMaxTN;
+  const int per = 1 + (T - 1) / d.token_tiles;
+  d.tn = (per + 31) / 32 * 32;
+  const int items = lm_units(V, kw) * d.token_tiles;
+  const int left = items % pairs;
+  const int halved = kw == 2 && 2 * left <= pairs ? left : 0;
+  d.full = items - halved;
+  d.entries = items + halved;
+  return d;
+}
+
+}  // namespace asd_detail

@@ -18,7 +18,7 @@
 // rows cross from L2 once per two vocabulary tiles; with one token tile an item is
 // one vocabulary tile (see launch_lmhead). Items are dealt to the pairs in one
 // sequence, token tiles innermost, so the pairs that need a W row run at the
-// same time and it comes from HBM about once (see LmParams for the last round).
+// same time and it comes from HBM about once (see LmDeal for the last round).
 // Per CTA: warp 0 issues TMA loads (128B-swizzled 64-wide K slabs) into a ring
 // of as many stages as fit, whose completion is counted on the first CTA's
 // barrier; warp 1 allocates tensor memory, and in the first CTA one of its
@@ -41,15 +41,14 @@
 
 #include "asd.h"
 #include "asd_device.cuh"
+#include "asd_lm_deal.h"
 #include "asd_select.cuh"
 
 namespace {
 
 using namespace asd_detail;
 
-constexpr int kPairM = 256;               // vocabulary rows per CTA pair in one MMA (MMA M)
 constexpr int kHalfM = 128;               // vocabulary rows per CTA in one MMA (TMEM lanes)
-constexpr int kMaxTN = 256;               // most token rows per tile (MMA N; a multiple of 32)
 constexpr int kBK = 64;                   // K per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int kUmmaK = 16;                // K per tcgen05.mma (kind::f16)
 constexpr int kMaxStages = 12;
@@ -407,10 +406,7 @@ struct LmParams {
   int stages;       // ring stages
   int slots;        // accumulator slots
   int k_steps;      // ceil(H / kBK)
-  // Items 0 .. full - 1: item i is vocabulary rows (i / token_tiles) * kw * kPairM on by token tile i % token_tiles.
-  // When the last round of the deal would leave more than half of the pairs idle, its items are dealt in
-  // halves (one vocabulary tile each): entries full + 2 h and full + 2 h + 1 are the tiles of item full + h.
-  int full, entries;
+  int full, entries;  // of the deal
   float* logits_out;  // [T, V] when writing logits instead of verifying
 };
 
@@ -808,37 +804,24 @@ cudaLaunchConfig_t pair_config(unsigned grid, int threads, size_t smem, cudaStre
   return cfg;
 }
 
-// How T token rows and V vocabulary rows are cut and dealt to `pairs` CTA pairs.
-//
-// Token tiles: as few as hold T at up to 256 columns (each tile reads W once
-// more from L2, and a wider MMA reads its vocabulary operand from shared memory
-// less often per product), all of one width, rounded up to the 32 columns of an
-// epilogue block. Against a fixed width of 192: 320 rows took 384 columns and
-// take 2 x 160, 18 rows take 32, 2304 rows take 9 tiles instead of 12.
-//
-// The last round of the deal: `left` items for more pairs. Up to half of the
-// pairs' number, half items keep twice as many pairs busy for half the time;
-// beyond that, halves would only begin a second round.
-void lm_plan(int T, int V, int H, int kw, int pairs, LmParams* q) {
-  q->T = T;
-  q->H = H;
-  q->V = V;
-  q->token_tiles = (T + kMaxTN - 1) / kMaxTN;
-  const int per = (T + q->token_tiles - 1) / q->token_tiles;
-  q->tn = (per + 31) / 32 * 32;
-  q->stages = lm_stages(q->tn, kw);
-  q->slots = kTmemCols / q->tn < kMaxSlots ? kTmemCols / q->tn : kMaxSlots;
-  q->k_steps = (H + kBK - 1) / kBK;
-  const int unit = kw * kPairM;
-  const int items = (V + unit - 1) / unit * q->token_tiles;
-  const int left = items % pairs;
-  const int halved = kw == 2 && 2 * left <= pairs ? left : 0;
-  q->full = items - halved;
-  q->entries = items + halved;
+LmParams lm_params(int T, int V, int H, int kw, int pairs) {
+  const LmDeal d = lm_deal(T, V, kw, pairs);
+  LmParams q = {};
+  q.T = T;
+  q.H = H;
+  q.V = V;
+  q.tn = d.tn;
+  q.token_tiles = d.token_tiles;
+  q.full = d.full;
+  q.entries = d.entries;
+  q.stages = lm_stages(d.tn, kw);
+  q.slots = kTmemCols / d.tn < kMaxSlots ? kTmemCols / d.tn : kMaxSlots;
+  q.k_steps = 1 + (H - 1) / kBK;
+  return q;
 }
 
 template <bool kWriteLogits, int kEpi, int kW>
-int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
+int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, const VerifyParams& p, float* logits_out,
                          cudaStream_t stream) {
   LmDevice* dev = nullptr;
   int rc = lm_device(&dev);
@@ -858,8 +841,7 @@ int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, V
     if (cudaOccupancyMaxActiveClusters(&pairs, kernel, &probe) != cudaSuccess || pairs < 1) return ASD_ERR_CUDA;
     resident.store(pairs, std::memory_order_release);
   }
-  LmParams q;
-  lm_plan(T, p.V, H, kW, pairs, &q);
+  LmParams q = lm_params(T, p.V, H, kW, pairs);
   q.logits_out = logits_out;
   CUtensorMap map_h, map_w;
   if (!make_map(&map_h, hidden, T, H, q.tn / 2) || !make_map(&map_w, weight, p.V, H, kHalfM)) return ASD_ERR_CUDA;
@@ -879,11 +861,42 @@ int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, V
 // instead of 226.5 / 227 / 229 / 249.5. With several token tiles the tensor cores
 // set the pace, and two vocabulary tiles per token slab feed them with less.
 template <bool kWriteLogits>
-int launch_lmhead(const void* hidden, const void* weight, int H, int T, VerifyParams& p, float* logits_out,
+int launch_lmhead(const void* hidden, const void* weight, int H, int T, const VerifyParams& p, float* logits_out,
                   cudaStream_t stream) {
   if (T > kMaxTN) return launch_lmhead_kernel<kWriteLogits, kEpiWarps, 2>(hidden, weight, H, T, p, logits_out, stream);
   constexpr int kEpi = kWriteLogits ? kEpiWarps : kEpiWarpsOneTile;
   return launch_lmhead_kernel<kWriteLogits, kEpi, 1>(hidden, weight, H, T, p, logits_out, stream);
+}
+
+// Verify or partials of p.B requests, in as many launches as their rows need.
+int verify_lmhead(const void* hidden, const void* weight, int H, const VerifyParams& p, cudaStream_t stream) {
+  const int K1 = p.K + 1, most = lm_rows_per_launch(p.V) / K1;
+  for (long long b = 0; b < p.B; b += most) {
+    const long long row = b * K1;
+    VerifyParams c = p;
+    c.B = static_cast<int>(p.B - b < most ? p.B - b : most);
+    c.draft = p.draft + b * p.K;
+    c.row_key = p.row_key + row;
+    c.draft_logit = p.draft_logit + row;
+    c.done = p.done + b;
+    c.flags = p.flags + b;
+    if (p.partials) {
+      c.partials = p.partials + row;
+    } else {
+      c.ledger = p.ledger + b;
+      c.accepted_len = p.accepted_len + b;
+      c.committed = p.committed + row;
+      c.recovery = p.recovery + b;
+      if (p.row_argmax) c.row_argmax = p.row_argmax + row;
+      if (p.row_regret) c.row_regret = p.row_regret + b * p.K;
+      if (p.row_top) c.row_top = p.row_top + row;
+      if (p.status) c.status = p.status + b;
+    }
+    const int rc = launch_lmhead<false>(static_cast<const char*>(hidden) + 2 * row * H, weight, H, c.B * K1, c, nullptr,
+                                        stream);
+    if (rc != ASD_OK) return rc;
+  }
+  return ASD_OK;
 }
 
 int check_lm_inputs(const void* hidden, const void* weight, int H) {
@@ -946,8 +959,7 @@ int asd_lmhead_verify(const void* hidden, const void* weight, int H, int B, int 
   p.error = reinterpret_cast<unsigned int*>(ws + l.error);
   p.row_top = row_top;
   p.nblk = 1;
-  return launch_lmhead<false>(hidden, weight, H, B * (K + 1), p, nullptr,
-                                     reinterpret_cast<cudaStream_t>(stream));
+  return verify_lmhead(hidden, weight, H, p, reinterpret_cast<cudaStream_t>(stream));
 }
 
 int asd_lmhead_partials(const void* hidden, const void* weight, int H, int B, int K, int Vs, int v_offset,
@@ -981,8 +993,7 @@ int asd_lmhead_partials(const void* hidden, const void* weight, int H, int B, in
   p.v_offset = v_offset;
   p.v_total = V;
   p.partials = partials;
-  return launch_lmhead<false>(hidden, weight, H, B * (K + 1), p, nullptr,
-                                    reinterpret_cast<cudaStream_t>(stream));
+  return verify_lmhead(hidden, weight, H, p, reinterpret_cast<cudaStream_t>(stream));
 }
 
 int asd_lmhead_logits(const void* hidden, const void* weight, int H, int T, int V, float* logits,
@@ -996,7 +1007,14 @@ int asd_lmhead_logits(const void* hidden, const void* weight, int H, int T, int 
   p.V = V;
   p.K = 0;
   p.nblk = 1;
-  return launch_lmhead<true>(hidden, weight, H, T, p, logits, reinterpret_cast<cudaStream_t>(stream));
+  const int most = lm_rows_per_launch(V);
+  for (long long t = 0; t < T; t += most) {
+    rc = launch_lmhead<true>(static_cast<const char*>(hidden) + 2 * t * H, weight, H,
+                             static_cast<int>(T - t < most ? T - t : most), p, logits + t * V,
+                             reinterpret_cast<cudaStream_t>(stream));
+    if (rc != ASD_OK) return rc;
+  }
+  return ASD_OK;
 }
 
 }  // extern "C"

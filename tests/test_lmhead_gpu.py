@@ -9,6 +9,7 @@ every row has such a gap, every mismatch has |r/q - g| > 5e-2 and every
 budget test has |fl(s + C) - B| > 4e-2 per accumulated mismatch.
 """
 import concurrent.futures as cf
+import ctypes
 import math
 
 import numpy as np
@@ -16,7 +17,7 @@ import pytest
 import torch
 
 from oracle import oracle
-from paper_2608_03447_gb300 import inputs
+from paper_2608_03447_gb300 import build, inputs
 
 pytestmark = pytest.mark.gpu
 LOGIT_TOL = 2e-2
@@ -399,3 +400,30 @@ def test_lmhead_verify_infinities_through_the_tensor_cores(asd):
     assert np.array_equal(np.isnan(a), np.isnan(b))
     assert np.array_equal(a[~np.isnan(a)].view(np.int32), b[~np.isnan(b)].view(np.int32))
     assert np.array_equal(led.cpu().numpy().view(np.int32), o["ledger"].view(np.int32))
+
+
+def test_calls_of_several_launches(asd, tmp_path, monkeypatch):
+    """More items than a launch counts: the call takes several launches, each with its requests' slices of every
+    array. The limit (2^30 items) is lowered to four in a build of its own: 512 rows a launch."""
+    path = build.build(extra=["-DASD_LM_MAX_ITEMS=4"], output=str(tmp_path / "libasd_split.so"))
+    monkeypatch.setattr(asd, "_lib", asd._declare(ctypes.CDLL(path)))
+    B, K, H, V = 150, 8, 72, 1000
+    inp = inputs.gen_lmhead_exact(B, K, H, V, 7777, "cuda")
+    inp.draft[70, 3] = V
+    ledgers = [asd.make_ledger(B, 8.0) for _ in range(2)]
+    out = asd.lmhead_verify(inp.hidden, inp.weight, inp.draft, ledgers[0], 1.0, 2)
+    logits = asd.lmhead_logits(inp.hidden, inp.weight)
+    parts = torch.stack([asd.lmhead_partials(inp.hidden, inp.weight[lo:hi].contiguous(), inp.draft, lo, V)
+                         for lo, hi in ((0, 601), (601, V))])
+    combined = asd.shard_combine(parts, inp.draft, ledgers[1], 1.0, 2, V)
+    torch.cuda.synchronize()
+    z = oracle.lmhead_logits_matmul(inp.hidden.cpu(), inp.weight.cpu()).astype(np.float32)
+    assert np.array_equal(logits.cpu().numpy(), z)
+    o = oracle.verify(z.reshape(B, K + 1, V), inp.draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), 1.0, 2)
+    for got, ledger in ((out, ledgers[0]), (combined, ledgers[1])):
+        for key in ("accepted_len", "committed", "recovery", "row_argmax", "status"):
+            assert np.array_equal(got[key].cpu().numpy(), o[key]), key
+        g, w = got["row_regret"].cpu().numpy(), o["row_regret"]
+        assert ((g.view(np.uint32) == w.view(np.uint32)) | (np.isnan(g) & np.isnan(w))).all()
+        assert np.array_equal(ledger.cpu().numpy().view(np.uint32), o["ledger"].view(np.uint32))
+    assert np.array_equal(out["row_top"].cpu().numpy().reshape(-1), z.max(axis=1))
