@@ -53,3 +53,13 @@ def test_items_of_a_launch_fit_32_bits(lib, T, V):
         assert full <= items <= entries <= 2**31 - 1 - 76
         assert full + (entries - full) // (1 if entries == items else 2) == items
         assert (entries - full) % 2 == 0 or entries == full
+
+
+@pytest.mark.parametrize("T,V,tiles,tn", [
+    (477, 12800, 3, 160), (477, 12801, 2, 256),     # 75 items of three tiles are one round, 78 are not
+    (477, 9728, 2, 256), (477, 9729, 3, 160),       # 38 items go in halves, 40 do not
+    (600, 9717, 4, 160), (600, 9729, 3, 224),       # 76 and 80 items
+    (300, 12509, 2, 160), (384, 12509, 2, 192), (385, 12509, 3, 160),
+    (2304, 151936, 9, 256), (576, 151936, 3, 192)])
+def test_one_round_of_narrower_tiles(lib, T, V, tiles, tn):
+    assert _deal(lib, T, V, 2)[:2] == (tn, tiles)

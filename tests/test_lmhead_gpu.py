@@ -230,7 +230,9 @@ def test_lmhead_full_size_exact_inputs_bit_exact(asd):
 # lies past the vocabulary, of whole items (76 + 39), and one partial item; one, three and eight K steps.
 @pytest.mark.parametrize("B,K,H,V", [(1, 0, 8, 39424), (4, 7, 136, 39424), (33, 0, 512, 39000), (32, 7, 136, 39040),
                                      (257, 0, 72, 39424), (16, 9, 136, 58700), (32, 8, 72, 19456), (27, 18, 72, 13100),
-                                     (64, 9, 72, 600)])
+                                     (64, 9, 72, 600)]
+                         # one round of narrower tiles and both sides of it
+                         + [(53, 8, 136, 12509), (60, 9, 72, 9717), (55, 6, 72, 12801)])
 def test_lmhead_token_tiles_and_deal_exact_inputs(asd, B, K, H, V):
     inp = inputs.gen_lmhead_exact(B, K, H, V, 7900 + B + K + H, "cuda")
     T = B * (K + 1)
