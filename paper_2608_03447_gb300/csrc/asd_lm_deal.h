@@ -66,4 +66,14 @@ inline LmDeal lm_deal(int T, int V, int kw, int pairs) {
   return d;
 }
 
+// Logits of one token tile: items of two vocabulary tiles where items of one would
+// begin a second round with few of them. On 19500 to 24000 vocabulary rows, H = 3000,
+// 109 rows 31.8-37.2 -> 28.9-31.4 us, 250 rows 41.6-48.1 -> 37.9-40.9; a fuller second
+// round gains nothing (32000 rows, H = 5120: 57.0 against 58.3), nor does the verify,
+// which stores nothing (250 rows, H = 5120: 58.2 against 59.5 us).
+inline bool lm_logits_in_two_tiles(int V, int pairs) {
+  const int units = lm_units(V, 1);
+  return units > pairs && units <= pairs + pairs / 4;
+}
+
 }  // namespace asd_detail

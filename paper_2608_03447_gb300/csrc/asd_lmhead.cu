@@ -821,11 +821,8 @@ LmParams lm_params(int T, int V, int H, int kw, int pairs) {
 }
 
 template <bool kWriteLogits, int kEpi, int kW>
-int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, const VerifyParams& p, float* logits_out,
-                         cudaStream_t stream) {
-  LmDevice* dev = nullptr;
-  int rc = lm_device(&dev);
-  if (rc != ASD_OK) return rc;
+int launch_lmhead_kernel(LmDevice* dev, const void* hidden, const void* weight, int H, int T, const VerifyParams& p,
+                         float* logits_out, cudaStream_t stream) {
   if (dev->major != 10) return ASD_ERR_DEVICE;  // tcgen05 needs a Blackwell (sm_10x) device
   auto kernel = lmhead_verify_kernel<kWriteLogits, kEpi, kW>;
   std::atomic<int>& resident = dev->pairs[2 * (kW - 1) + (kWriteLogits ? 1 : 0)];
@@ -863,9 +860,13 @@ int launch_lmhead_kernel(const void* hidden, const void* weight, int H, int T, c
 template <bool kWriteLogits>
 int launch_lmhead(const void* hidden, const void* weight, int H, int T, const VerifyParams& p, float* logits_out,
                   cudaStream_t stream) {
-  if (T > kMaxTN) return launch_lmhead_kernel<kWriteLogits, kEpiWarps, 2>(hidden, weight, H, T, p, logits_out, stream);
+  LmDevice* dev = nullptr;
+  const int rc = lm_device(&dev);
+  if (rc != ASD_OK) return rc;
+  if (T > kMaxTN || (kWriteLogits && lm_logits_in_two_tiles(p.V, dev->sms / 2)))
+    return launch_lmhead_kernel<kWriteLogits, kEpiWarps, 2>(dev, hidden, weight, H, T, p, logits_out, stream);
   constexpr int kEpi = kWriteLogits ? kEpiWarps : kEpiWarpsOneTile;
-  return launch_lmhead_kernel<kWriteLogits, kEpi, 1>(hidden, weight, H, T, p, logits_out, stream);
+  return launch_lmhead_kernel<kWriteLogits, kEpi, 1>(dev, hidden, weight, H, T, p, logits_out, stream);
 }
 
 // Verify or partials of p.B requests, in as many launches as their rows need.

@@ -16,6 +16,7 @@ extern "C" void deal(int T, int V, int kw, int pairs, int* out) {
   out[3] = d.entries;
 }
 extern "C" int rows_per_launch(int V) { return asd_detail::lm_rows_per_launch(V); }
+extern "C" int logits_in_two_tiles(int V, int pairs) { return asd_detail::lm_logits_in_two_tiles(V, pairs); }
 """
 
 
@@ -63,3 +64,7 @@ def test_items_of_a_launch_fit_32_bits(lib, T, V):
     (2304, 151936, 9, 256), (576, 151936, 3, 192)])
 def test_one_round_of_narrower_tiles(lib, T, V, tiles, tn):
     assert _deal(lib, T, V, 2)[:2] == (tn, tiles)
+
+
+def test_logits_of_one_tile(lib):
+    assert [lib.logits_in_two_tiles(V, 76) for V in (19456, 19457, 24320, 24321, 151936)] == [0, 1, 1, 0, 0]

@@ -231,8 +231,10 @@ def test_lmhead_full_size_exact_inputs_bit_exact(asd):
 @pytest.mark.parametrize("B,K,H,V", [(1, 0, 8, 39424), (4, 7, 136, 39424), (33, 0, 512, 39000), (32, 7, 136, 39040),
                                      (257, 0, 72, 39424), (16, 9, 136, 58700), (32, 8, 72, 19456), (27, 18, 72, 13100),
                                      (64, 9, 72, 600)]
-                         # one round of narrower tiles and both sides of it
-                         + [(53, 8, 136, 12509), (60, 9, 72, 9717), (55, 6, 72, 12801)])
+                         # one round of narrower tiles and both sides of it; logits of one token tile in items of two
+                         # vocabulary tiles, whole, halved and with a second tile past the vocabulary
+                         + [(53, 8, 136, 12509), (60, 9, 72, 9717), (55, 6, 72, 12801), (9, 8, 136, 19457),
+                            (32, 7, 72, 24320), (1, 0, 72, 20000), (25, 4, 72, 24321)])
 def test_lmhead_token_tiles_and_deal_exact_inputs(asd, B, K, H, V):
     inp = inputs.gen_lmhead_exact(B, K, H, V, 7900 + B + K + H, "cuda")
     T = B * (K + 1)
