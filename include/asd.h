@@ -365,7 +365,8 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches);
  *   path          ASD_PATH_AUTO picks the row-stage kernel by size (one CTA or
  *                 one cluster of CTAs per request, selection included, for few
  *                 requests that fit it; the TMA pipeline for
- *                 ASD_RESIDENT_INPUTS in long rows (few, or more than 21 MB);
+ *                 ASD_RESIDENT_INPUTS in long rows (few, or more than 21 MB)
+ *                 and, with fused_select, for more than 80 MB in long rows;
  *                 the register-streaming kernel for everything else); the
  *                 others force one (a forced ASD_PATH_SMALL falls back to AUTO
  *                 where the shape does not fit it).

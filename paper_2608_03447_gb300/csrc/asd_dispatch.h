@@ -59,6 +59,10 @@ constexpr int kMeasuredSms = 152;
 //            nothing to overlap and takes 14.8-15.1 us for 87.5 MB where the TMA
 //            pipeline took 20.5 us, 91.7 against 100 us for 662 MB, 3.6 against
 //            8.2 us for 2.7 MB, 7 against 26 us for 16 MB in 2 KB rows.
+// With the selection inside the row stage (a launch option) the streaming kernel's
+// CTAs each fence and count their units, the pipeline's a slice: 15.4 against 18.4 us
+// at 43 MB, but 24.5 against 23.5 at 86 MB with 200 KB rows, 146 against 102 at 659 MB
+// with 304 KB rows; with 64 KB rows 129 against 140 us.
 // The launch options can force a kernel (the tests use that to cover every
 // kernel); a forced `small` falls back to the default when the shape does not
 // qualify.
@@ -68,6 +72,8 @@ constexpr long long kTmaFewRows = 64;
 constexpr long long kTmaMinRowBytes = 64LL << 10;        // up to kTmaManyRows
 constexpr long long kTmaMinRowBytesManyRows = 112LL << 10;
 constexpr long long kTmaManyRows = 3;                    // a slice, of which there is one a SM
+constexpr long long kFusedTmaMinBytes = 80LL * 1000 * 1000;
+constexpr long long kFusedTmaMinRowBytes = 192LL << 10;
 constexpr long long kSmallMaxBytes = 1LL << 20;         // below this as many one-CTA requests as fit at once
 constexpr int kSmallWarpsPerSm = 22;                    // at 88 registers a thread
 constexpr long long kSmallMaxClusterBytes = 5LL << 20;  // of clusters larger than two
@@ -108,7 +114,7 @@ inline SmallPlan small_plan(int nvec, int K, int ctas) {
 }
 
 inline Path choose_path(int forced, long long bytes, long long request_bytes, int B, int K, bool single_block,
-                        bool resident, int sms) {
+                        bool resident, bool fused, int sms) {
   const int ctas = single_block ? small_cluster(request_bytes) : 0;
   if (forced == ASD_PATH_TMA) return Path::kTma;
   if (forced == ASD_PATH_STREAM) return Path::kStream;
@@ -124,6 +130,7 @@ inline Path choose_path(int forced, long long bytes, long long request_bytes, in
   if (resident && bytes >= (rows <= kTmaFewRows ? kTmaMinBytesFewRows : kTmaMinBytes * sms / kMeasuredSms) &&
       row_bytes >= (rows <= kTmaManyRows * sms ? kTmaMinRowBytes : kTmaMinRowBytesManyRows))
     return Path::kTma;
+  if (fused && bytes >= kFusedTmaMinBytes && row_bytes >= kFusedTmaMinRowBytes) return Path::kTma;
   return Path::kStream;
 }
 

@@ -1103,7 +1103,7 @@ int launch(VerifyParams& p, cudaStream_t stream) {
   const long long request_bytes = static_cast<long long>(p.K + 1) * p.V * static_cast<long long>(sizeof(T));
   const LaunchOptions opt = launch_options();
   const Path path = choose_path(opt.path, p.total * static_cast<long long>(sizeof(T)), request_bytes, p.B, p.K,
-                                p.nblk == 1 && !p.partials, p.resident != 0, info->sms);
+                                p.nblk == 1 && !p.partials, p.resident != 0, !opt.split, info->sms);
   const long long head = static_cast<long long>(((16 - addr % 16) % 16) / sizeof(T));
   p.head = head < p.total ? head : p.total;
   if (path == Path::kTma) return launch_tma<T, kStrict>(p, info, opt, stream);
@@ -1241,8 +1241,8 @@ int asd_verify_launches(int B, int K, int V, int dtype, int* launches) {
     sms = info->sms;
   else
     cudaGetLastError();  // not the caller's
-  const Path path =
-      choose_path(opt.path, request_bytes * B, request_bytes, B, K, true, (dtype & ASD_RESIDENT_INPUTS) != 0, sms);
+  const Path path = choose_path(opt.path, request_bytes * B, request_bytes, B, K, true,
+                                (dtype & ASD_RESIDENT_INPUTS) != 0, !opt.split, sms);
   *launches = B == 0 ? 0 : (path != Path::kSmall && opt.split ? 2 : 1);
   return ASD_OK;
 }

@@ -13,9 +13,10 @@ KB, MB = 1 << 10, 1 << 20
 
 SHIM = """
 #include "asd_dispatch.h"
-extern "C" int path_of(int B, int K, int row_bytes, int single, int resident, int sms) {
+extern "C" int path_of(int B, int K, int row_bytes, int single, int resident, int fused, int sms) {
   const long long request = static_cast<long long>(K + 1) * row_bytes;
-  return static_cast<int>(asd_detail::choose_path(ASD_PATH_AUTO, request * B, request, B, K, single, resident, sms));
+  return static_cast<int>(asd_detail::choose_path(ASD_PATH_AUTO, request * B, request, B, K, single, resident, fused,
+                                                  sms));
 }
 """
 
@@ -28,8 +29,8 @@ def path_of(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", f"-I{build.INCLUDE}",
                     f"-I{build.CSRC}", str(d / "shim.cpp"), "-o", out], check=True)
     lib = ctypes.CDLL(out)
-    return lambda B, K, row_bytes, single=True, resident=False, sms=152: lib.path_of(
-        B, K, row_bytes, int(single), int(resident), sms)
+    return lambda B, K, row_bytes, single=True, resident=False, fused=False, sms=152: lib.path_of(
+        B, K, row_bytes, int(single), int(resident), int(fused), sms)
 
 
 @pytest.mark.parametrize("sms", [152, 76])
@@ -90,3 +91,14 @@ def test_few_long_rows_go_to_the_tma_pipeline_from_a_megabyte_on(path_of):
     assert path_of(1, 1, 512 * KB, resident=True) == TMA          # 1 MB
     assert path_of(1, 0, MB - 16, resident=True) == STREAM
     assert path_of(13, 4, 64 * KB, resident=True, single=False) == STREAM  # 65 rows, 4 MB
+
+
+def test_selection_inside_the_row_stage(path_of):
+    """Large calls in long rows take the pipeline, whose CTAs count slices; without it they do not."""
+    row = 192 * KB
+    B = 80_000_000 // (9 * row)
+    assert path_of(B + 1, 8, row, fused=True) == TMA
+    assert path_of(B, 8, row, fused=True) == STREAM
+    assert path_of(B + 1, 8, row - 16, fused=True) == STREAM
+    assert path_of(B + 1, 8, row) == STREAM
+    assert path_of(1, 8, KB, fused=True) == SMALL
