@@ -3,8 +3,9 @@ block of a request, every block checked against the oracle bit for bit (Alg. 1's
 ledger, the row argmaxes and fp32 regrets).
 
   * Qwen3-14B-shaped verify (B=32, K=8, V=151936 bf16, g=1, M=2, budget 8): 256 sequential blocks, through
-    the default launch (the row stage waits for the previous kernel), with resident inputs (overlapping
-    launches), with the selection inside the row stage, and through the register-streaming kernel;
+    the default launch (the streaming row stage waits for the previous kernel), with resident inputs (the
+    TMA row stage, overlapping launches), and through the TMA row stage of a waiting call, with its
+    selection behind it and inside it;
   * large-batch serving shape (B=256, K=4, V=129280, g=1, M=1, budget 4): 64 blocks at each of the four
     acceptance points, fp32 and bf16, with and without resident inputs;
   * the benchmark's launch configuration: 256 steps over its rotating buffers captured in one CUDA graph,
@@ -129,7 +130,7 @@ def long_run(asd, B, K, V, dtype, nblocks, gate, cap, budget, config, variants, 
 DEFAULT = ({}, False)
 RESIDENT = ({}, True)
 FUSED = ({"path": "tma", "fused_select": True}, False)
-STREAM = ({"path": "stream"}, False)
+WAITING_TMA = ({"path": "tma"}, False)
 
 
 def test_qwen3_shape_256_carried_blocks(asd):
@@ -137,7 +138,7 @@ def test_qwen3_shape_256_carried_blocks(asd):
     cfg = inputs.CONFIGS[1]
     expect = long_run(asd, cfg["B"], cfg["K"], cfg["V"], cfg["dtype"], 256, cfg["gate"], cfg["cap"],
                       cfg["budget"], 1, {"default": DEFAULT, "resident": RESIDENT, "fused": FUSED,
-                                         "stream": STREAM})
+                                         "waiting tma": WAITING_TMA})
     spent = expect[-1]["ledger"][:, 1]
     assert np.all(spent <= cfg["budget"])
     assert np.all(spent > 0), "every request should have spent some of its budget over 256 blocks"
@@ -217,8 +218,8 @@ def test_bench_graph_every_step_matches_oracle(asd, resident):
 
 @pytest.mark.parametrize("path", ["auto", "stream"])
 def test_more_than_2_31_logits(asd, path):
-    """B=1600, K=8, V=151936 bf16: 2.19e9 logits (4.4 GB), past every 32-bit element offset. The TMA row
-    stage (with and without resident inputs) and the register-streaming kernel match the oracle, which
+    """B=1600, K=8, V=151936 bf16: 2.19e9 logits (4.4 GB), past every 32-bit element offset. The streaming row
+    stage (waiting, and with resident inputs) and the TMA row stage (with resident inputs) match the oracle, which
     runs request slices in parallel (requests are independent; each slice carries its own ledgers)."""
     B, K, V = 1600, 8, 151936
     assert B * (K + 1) * V > 2**31

@@ -1,5 +1,5 @@
 """The row stages that cut rows into units, at the sizes where the cut can go wrong: one vector either side of
-a unit, a unit of one, four and eight loads per lane, rows shorter than a vector, starts off the 16-byte and the
+a unit, units of one to eight loads per lane, rows shorter than a vector, starts off the 16-byte and the
 128-byte grid, rows whose maximum sits at a unit's edge or is tied across units, rows of -inf, infinities, the
 lowest finite value and subnormal maxima; requests on both sides of each cluster size; several blocks per call.
 Every output bit for bit the oracle's (comparisons and one fp32 subtraction decide all of them)."""
@@ -61,6 +61,42 @@ def test_unit_edges(asd, dtype, vectors, fused):
             asd.reset_launch_options()
         want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), 1.0, 2)
         _equal(out, want, f"V={V} off={off} {dtype}")
+        assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("per", [64, 96, 128, 160, 192, 224])
+@pytest.mark.parametrize("units", [1, 2, 3])
+def test_units_of_several_loads(asd, per, units, dtype):
+    """Inputs whose size gives units of `per` vectors (sixteen warps an SM share them), in rows one vector either
+    side of a whole number of them."""
+    vn, K = VEC[dtype], 3
+    warps = 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    for vectors in (per * units - 1, per * units, per * units + 1, per * units - 7, per * units - 8):
+        B = max(3, int(warps * (per - 16) / vectors) // (K + 1))
+        share = -(-B * (K + 1) * vectors // warps)
+        assert -(-share // 32) * 32 == per
+        V = vectors * vn + vectors % vn
+        off = vectors % 61
+        flat = torch.randn(off + B * (K + 1) * V, device="cuda").mul_(3.0).to(dtype)
+        z = flat[off:].view(B, K + 1, V)
+        for i in range(min(B, 40)):
+            edge = (i % (units + 1)) * per * vn
+            at = [edge - 8 * vn, edge - 1, edge, edge + vn]
+            for j in range(K + 1):
+                z[i, j, min(max(at[j], 0), V - 1)] = 40.0
+        z[2, 1, [0, V - 1]] = 50.0
+        draft = torch.randint(0, V, (B, K), dtype=torch.int32, device="cuda")
+        draft[:, 0] = z[:, 0].argmax(1)
+        ledger = asd.make_ledger(B, 8.0)
+        try:
+            asd.set_launch_options(path="stream")
+            out = asd.verify(z, draft, ledger, 1.0, 2)
+            torch.cuda.synchronize()
+        finally:
+            asd.reset_launch_options()
+        want = oracle.verify(z.cpu(), draft.cpu().numpy(), np.array([[8.0, 0.0]] * B, np.float32), 1.0, 2)
+        _equal(out, want, f"per={per} V={V} off={off} {dtype}")
         assert np.array_equal(ledger.cpu().numpy().view(np.uint32), want["ledger"].view(np.uint32))
 
 

@@ -485,15 +485,17 @@ def test_launches_without_programmatic_dependent_launch(asd, shape):
 
 
 def test_concurrent_streams_keep_their_own_state(asd):
-    """Three streams issue dependent sequences at the same time, interleaved call by call and never
-    synchronised with each other: the TMA row stage with its selection kernel (Qwen3-14B shape), the
+    """Four streams issue dependent sequences at the same time, interleaved call by call and never
+    synchronised with each other: the TMA row stage (Qwen3-14B shape, resident inputs) and the streaming
+    one (the same shape, each call waiting), both with the selection kernel behind them, the
     one-CTA-per-request kernel (the tiny shape), and the fused LM-head verify (exact inputs). Each
     stream has its own workspace and ledger; every call equals the oracle, so no call sees another
     stream's state."""
     n = 5
-    specs = [(32, 8, 151936, torch.bfloat16), (4, 8, 1024, torch.float32)]
+    specs = [(32, 8, 151936, torch.bfloat16, True), (32, 8, 151936, torch.bfloat16, False),
+             (4, 8, 1024, torch.float32, False)]
     seqs = []
-    for s, (B, K, V, dtype) in enumerate(specs):
+    for s, (B, K, V, dtype, resident) in enumerate(specs):
         blocks = [inputs.gen_block(B, K, V, dtype, 9400 + 10 * s + i, "cuda") for i in range(n)]
         led = np.array([[4.0, 0.0]] * B, np.float32)
         expect = []
@@ -501,7 +503,7 @@ def test_concurrent_streams_keep_their_own_state(asd):
             o = oracle.verify(b.logits.cpu(), b.draft.cpu().numpy(), led, 1.0, 2)
             expect.append(o)
             led = o["ledger"]
-        seqs.append(dict(blocks=blocks, expect=expect, ledger=asd.make_ledger(B, 4.0),
+        seqs.append(dict(blocks=blocks, expect=expect, ledger=asd.make_ledger(B, 4.0), resident=resident,
                          ws=asd.Workspace(B, K, V, asd.BF16 if dtype == torch.bfloat16 else asd.F32),
                          outs=[asd.alloc_outputs(B, K) for _ in range(n)], stream=torch.cuda.Stream()))
     Bl, Kl, Hl, Vl = 8, 8, 256, 1300
@@ -516,13 +518,13 @@ def test_concurrent_streams_keep_their_own_state(asd):
     lm_ws = asd.lmhead_workspace(Bl, Kl, Vl, Hl, torch.device("cuda"))
     lm_outs = [asd.alloc_outputs(Bl, Kl) for _ in range(n)]
     lm_stream = torch.cuda.Stream()
-    for st in [q["stream"] for q in seqs] + [lm_stream]:
-        st.wait_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()  # every input is written: resident calls may read ahead of what they are queued behind
     for i in range(n):
         for q in seqs:
             with torch.cuda.stream(q["stream"]):
                 b = q["blocks"][i]
-                asd.verify(b.logits, b.draft, q["ledger"], 1.0, 2, workspace=q["ws"], out=q["outs"][i])
+                asd.verify(b.logits, b.draft, q["ledger"], 1.0, 2, workspace=q["ws"], out=q["outs"][i],
+                           resident=q["resident"])
         with torch.cuda.stream(lm_stream):
             asd.lmhead_verify(lm[i].hidden, lm[i].weight, lm[i].draft, lm_led, 1.0, 2, workspace=lm_ws,
                               out=lm_outs[i])
