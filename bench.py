@@ -54,8 +54,8 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 # the sources each profiled kernel is built from (a recorded traffic figure is
 # reported only while these are unchanged)
 KERNEL_SOURCES = {
-    "verify_tma_kernel": ["asd_verify.cu", "asd_device.cuh"],
-    "lmhead_verify_kernel": ["asd_lmhead.cu", "asd_device.cuh"],
+    "verify_tma_kernel": ["asd_verify.cu", "asd_device.cuh", "asd_dispatch.h", "asd_select.cuh"],
+    "lmhead_verify_kernel": ["asd_lmhead.cu", "asd_device.cuh", "asd_lm_deal.h", "asd_select.cuh"],
 }
 LM_B, LM_K, LM_H, LM_V = 64, 8, 5120, 151936
 LM_WORKLOAD = "fused-lmhead: B=64 requests, K=8 (576 target rows), H=5120, V=151936, bf16 h and W, fp32 " \
