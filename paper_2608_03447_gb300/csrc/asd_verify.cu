@@ -971,9 +971,10 @@ int launch_tma(const VerifyParams& p, DeviceInfo* info, const LaunchOptions& opt
   constexpr long long kMinPerCta = 2LL * kTmaChunkBytes / static_cast<long long>(sizeof(T));
   const long long bulk = (p.total - p.head) / VN * VN;
   const bool split = opt.split;
-  const int slot = (sizeof(T) == 2 ? 2 : 0) + (kStrict ? 1 : 0) + (split ? 4 : 0);
+  // strictness is the selection's: one split instance for both
+  const int slot = (sizeof(T) == 2 ? 2 : 0) + (split ? 4 : kStrict ? 1 : 0);
   if (!info->tma_ready[slot].load(std::memory_order_acquire)) {
-    auto kernel = split ? verify_tma_kernel<T, kStrict, true> : verify_tma_kernel<T, kStrict, false>;
+    auto kernel = split ? verify_tma_kernel<T, false, true> : verify_tma_kernel<T, kStrict, false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(sizeof(TmaShared))) != cudaSuccess)
       return ASD_ERR_CUDA;
@@ -1010,7 +1011,7 @@ int launch_tma(const VerifyParams& p, DeviceInfo* info, const LaunchOptions& opt
       return ASD_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
   }
-  if (cudaLaunchKernelEx(&cfg, verify_tma_kernel<T, kStrict, true>, p, bulk_end, per_cta) != cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, verify_tma_kernel<T, false, true>, p, bulk_end, per_cta) != cudaSuccess)
     return ASD_ERR_CUDA;
   return launch_select<T, kStrict>(p, opt.pdl, stream);
 }
@@ -1061,8 +1062,9 @@ int launch_stream(const VerifyParams& p, DeviceInfo* info, const LaunchOptions& 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
   }
-  auto kernel = q.per <= 32 * kStreamUnrollSmall ? verify_stream_kernel<T, kStrict, kSplit, kStreamUnrollSmall>
-                                                 : verify_stream_kernel<T, kStrict, kSplit, kStreamUnroll>;
+  constexpr bool kSelectsStrict = kStrict && !kSplit;  // strictness is the selection's: one split instance for both
+  auto kernel = q.per <= 32 * kStreamUnrollSmall ? verify_stream_kernel<T, kSelectsStrict, kSplit, kStreamUnrollSmall>
+                                                 : verify_stream_kernel<T, kSelectsStrict, kSplit, kStreamUnroll>;
   if (cudaLaunchKernelEx(&cfg, kernel, p, q) != cudaSuccess) return ASD_ERR_CUDA;
   if (kSplit) return launch_select<T, kStrict>(p, opt.pdl, stream);
   return cudaGetLastError() == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
