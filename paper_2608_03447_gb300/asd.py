@@ -164,8 +164,8 @@ _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 def _stream(stream) -> int:
     if stream is None:
-        # the handle of torch.cuda.current_stream() without building a Stream object around it, which took
-        # 2.9 us of an eager call's 12.4 us
+        # the handle of torch.cuda.current_stream() without building a Stream object around it: 2.9 us of an eager
+        # call's 12.4 us (8.7 us with load() answering before its lock, too)
         if _raw_stream is not None:
             return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()

@@ -30,8 +30,9 @@ struct VerifyParams {
   float* row_regret;
   int32_t* status;
   unsigned long long* row_key;  // [B*(K+1)] running (value, index) key, zero between calls
-  float* draft_logit;           // [B*(K+1)] z_j(x_j), written by the segment holding x_j
-  unsigned long long* done;     // [B] elements finished, zero between calls
+  float* draft_logit;           // [B*(K+1)] z_j(x_j), zero between calls
+  unsigned long long* done;     // [B] what a row stage that selects counts up to a request's completion (elements,
+                                // and in the streaming kernel each row's draft logit), zero between calls
   unsigned int* flags;          // [nblk*B] ASD_STATUS_NAN_LOGIT bits, zero between calls
   unsigned int* error;          // sticky: ASD_ERR_TIMEOUT when a pipeline wait gave up
   float* row_top;               // [B*(K+1)] z_j(y*_j), or NULL (written by the fused LM-head path)

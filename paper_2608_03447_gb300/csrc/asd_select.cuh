@@ -1,11 +1,12 @@
 // The selection as kernels of their own, launched right behind a row stage: the
-// TMA row stage of asd_verify.cu and the fused LM head of asd_lmhead.cu.
+// streaming and the TMA row stage of asd_verify.cu (which is also how a shard's rows
+// become partials) and the fused LM head of asd_lmhead.cu.
 //
-// One warp per request. It is launched with programmatic dependent launch and
-// small enough to fit beside the row stage's CTAs on an SM; griddepcontrol.wait
-// returns once the row stage has completed and its writes are visible, so no
-// counters and no fences are needed, and the row stage's CTAs leave their SMs
-// as soon as they have merged their rows.
+// One warp per request, or with several blocks one CTA. It is launched with
+// programmatic dependent launch and small enough to fit beside the row stage's
+// CTAs on an SM; griddepcontrol.wait returns once the row stage has completed and
+// its writes are visible, so no counters and no fences are needed, and the row
+// stage's CTAs leave their SMs as soon as they have merged their rows.
 #pragma once
 
 #include <cuda_runtime.h>

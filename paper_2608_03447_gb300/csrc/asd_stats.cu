@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kStatThreads)
   for (int i = threadIdx.x; i <= ncount; i += blockDim.x) local[i] = 0u;
   // programmatic dependent launch: the next kernel may start its set-up now;
   // this one reads the verify outputs only once the kernel before it is done,
-  // and past L1, which an earlier call of this kernel may have filled meanwhile
+  // each word once and so past L1
   pdl_signal_dependents();
   pdl_wait_prerequisites();
   __syncthreads();
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kCommitThreads) commit_kernel(int B, int K, co
   // a plain launch ended the chain, and a verify on resident inputs behind it
   // could not stream while the step before finished: 28.8 -> 12.6 us per step of
   // verify + opportunity + commit at B=32, K=8, V=151936 bf16 (12.0 verify
-  // alone). Loads go past L1: a line of it may be older than the kernel ahead.
+  // alone). Loads go past L1, which has nothing to give to words read once.
   pdl_signal_dependents();
   pdl_wait_prerequisites();
   const int lane = threadIdx.x & 31;

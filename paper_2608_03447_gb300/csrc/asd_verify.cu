@@ -15,11 +15,12 @@
 //              row j, resets the request's workspace slots to zero as it reads
 //              them, so the workspace is zero again after every call (whatever
 //              shape the next call has).
-// Three row-stage kernels (choose_path): verify_small_kernel (one CTA or cluster
+// Three row-stage kernels (asd_dispatch.h): verify_small_kernel (one CTA or cluster
 // per request, which selects it too) for few small requests, verify_stream_kernel
 // (one piece of one row per warp) for most calls, and verify_tma_kernel for
 // long rows declared resident. The latter two are followed by select_kernel
-// (or, as a launch option, select in the CTA that completes each request).
+// (several blocks: select_blocks_kernel) or, as a launch option, select in the
+// CTA that completes each request.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -933,7 +934,7 @@ std::atomic<int> g_flags{0};  // bit 0: selection inside the row stage, bit 1: n
 
 struct LaunchOptions {
   int path;
-  bool split;  // the TMA path's selection runs in select_kernel, right behind the row stage
+  bool split;  // the selection of the streaming and TMA paths runs in a kernel right behind the row stage
   bool pdl;    // launches carry the programmatic-serialization attribute
 };
 
