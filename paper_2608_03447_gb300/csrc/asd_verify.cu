@@ -921,7 +921,7 @@ __global__ void __launch_bounds__(kTmaThreads, ASD_TMA_MIN_BLOCKS)
 // ---------------------------------------------------------------- host side
 
 struct DeviceInfo {
-  int sms = 0;
+  std::atomic<int> sms = 0;  // 0: not asked yet; two threads racing to ask store the same value
   // set once the TMA kernel instance has its shared-memory opt-in; the
   // opt-in is idempotent, so two threads racing to set it up is harmless
   std::atomic<bool> tma_ready[8] = {};
@@ -952,15 +952,13 @@ LaunchOptions launch_options() {
 int device_info(DeviceInfo** info_out) {
   constexpr int kMaxDevices = 64;
   static DeviceInfo info[kMaxDevices];
-  static std::mutex mu;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return ASD_ERR_CUDA;
   if (dev < 0 || dev >= kMaxDevices) return ASD_ERR_DEVICE;
-  std::lock_guard<std::mutex> g(mu);
-  if (info[dev].sms == 0) {
+  if (info[dev].sms.load(std::memory_order_relaxed) == 0) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return ASD_ERR_CUDA;
-    info[dev].sms = sms;
+    info[dev].sms.store(sms, std::memory_order_relaxed);
   }
   *info_out = &info[dev];
   return ASD_OK;
@@ -985,8 +983,7 @@ int launch_tma(const VerifyParams& p, DeviceInfo* info, const LaunchOptions& opt
   // the SMs (one ramping up, one streaming, one finishing). Otherwise the
   // launch reads nothing before the previous kernel completes and runs alone,
   // so it fills every CTA slot of every SM itself.
-  const long long max_cta =
-      p.resident ? info->sms : static_cast<long long>(info->sms) * ASD_TMA_LONE_CTAS_PER_SM;
+  const long long max_cta = info->sms * (p.resident ? 1LL : ASD_TMA_LONE_CTAS_PER_SM);
   long long ncta = (bulk + kMinPerCta - 1) / kMinPerCta;
   if (ncta > max_cta) ncta = max_cta;
   if (ncta < 1) ncta = 1;
