@@ -260,7 +260,7 @@ int asd_verify_noalloc(const void* logits, int dtype, int B, int K, int V, const
  * row_regret    [nblk, B, K]
  * workspace     asd_blocks_workspace_size(nblk, B, K, V, dtype) bytes
  * The logits of all blocks stream in one pass; only each request's selection
- * runs block after block, with the ledger in registers.
+ * runs block after block, the ledger handed from one to the next.
  */
 int asd_blocks_workspace_size(int nblk, int B, int K, int V, int dtype, size_t* bytes);
 int asd_verify_blocks(const void* logits, int dtype, int nblk, int B, int K, int V,
