@@ -537,7 +537,7 @@ __device__ __forceinline__ uint4 lds128(const uint4* p) {
 }
 
 // Element `off` of a staged chunk, read with ld.shared (src is a shared-memory
-// pointer: the global-only loads of Elem<T>::load_cg must never see it).
+// pointer: the global-only loads of Elem<T> must never see it).
 __device__ __forceinline__ float smem_elem(const uint4* src, int off, float) {
   float v;
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(smem_u32(src) + 4u * static_cast<uint32_t>(off)));
@@ -589,7 +589,7 @@ __device__ __forceinline__ int draft_of_row(const VerifyParams& p, long long row
   const long long b = row / K1;
   const int j = static_cast<int>(row - b * K1);
   if (j >= p.K || b >= static_cast<long long>(p.B) * p.nblk) return -1;  // b: block-request
-  return __ldcg(p.draft + b * p.K + j) - p.v_offset;  // shard-local (no shift without a shard)
+  return p.draft[b * p.K + j] - p.v_offset;  // shard-local (no shift without a shard)
 }
 
 __device__ __forceinline__ void cursor_enter(RowCursor& c, const VerifyParams& p, long long row) {
@@ -743,7 +743,7 @@ __device__ __forceinline__ void consume_loose(RowCursor& c, const VerifyParams& 
     if (pos >= c.row1) cursor_advance<T>(c, p, sink, pos, lane);
     const long long seg_end = to < c.row1 ? to : c.row1;
     const long long e = pos + lane;
-    if (e < seg_end) lane_element(c, p, Elem<T>::load_cg(z, e), static_cast<int>(e - c.row0));
+    if (e < seg_end) lane_element(c, p, Elem<T>::load(z, e), static_cast<int>(e - c.row0));
     pos = seg_end;
   }
 }
