@@ -139,6 +139,8 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
 // wait -- most of them, most of the time -- take no issue slots from the MMA
 // and TMA threads (polling them cost this kernel about 7 %).
 constexpr uint32_t kSuspendNs = 1000000;
+// Longer than any load takes: what is waited, after a timeout, for loads that no barrier counts.
+constexpr unsigned long long kLandNs = 10000000;
 __device__ __forceinline__ bool mbar_try_wait_cluster(unsigned long long* bar, uint32_t parity) {
   uint32_t done;
   asm volatile(
@@ -716,6 +718,12 @@ __global__ void __launch_bounds__(lm_threads(kEpi), 1)
       const unsigned long long t0 = global_ns();
       while (!mbar_try_wait_cluster(&sh.full[issued_stage], issued_phase) && global_ns() - t0 < kWaitLimitNs) {
       }
+    }
+  }
+  if (sh.abort && !leader && warp == 0 && lane == 0) {
+    // the second CTA may be a load ahead of the first, whose barrier does not wait for that one: give it time to land
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < kLandNs) {
     }
   }
   __syncthreads();
